@@ -671,128 +671,205 @@ compact_fill_tc_kernel(ConvDims d, const uint4 *__restrict__ W0, const uint4 *__
   if (warp == 0) tc::tmem_dealloc(tmem, 64);
 }
 
-// Weight gradient  dW[cout][cin][tap] += sum over pixels of X[pixel + tap][cin] dY[pixel][cout]
-// as D[(tap, cin)][cout] = A[(tap, cin)][pixel] B[cout][pixel]^T with K = pixels: per 8 x 8
-// pixel tile the CTA transposes the halo into A (K-major, one M-tile per 128 (tap, cin) rows)
-// and dY into B, and accumulates in tensor memory over the tiles it owns; the bias gradient
-// is summed alongside.  Partial results are added to the fp32 outputs with atomics.
-constexpr int kWgTile = 8;   // 8 x 8 pixel tiles, K = 64 per tile
-
+// Weight gradient  dW[cout][cin][tap] += sum over pixels of X[q + tap][cin] dY[q][cout]  as one
+// accumulator  D[(ky, cout)][(kx, cin)] += A[(ky, cout)][pixel] B[(kx, cin)][pixel]^T  with K =
+// the pixels p of X: the row of A for tap row ky is dY one row below, at or above p, the row of B
+// for tap column kx is X one column left of, at or right of the column of dY.  Both operands are
+// read as they lie in memory, channels innermost (MN-major descriptors: a core matrix is 8 pixels
+// of one image row x 8 channels, 16 bytes a pixel), so a tile is staged by 16-byte asynchronous
+// copies alone and nothing is transposed:
+//   dY as [row][cout group][column]: the rows are 8 COUT / 8 core matrices apart, so the M groups
+//      (2 - ky, cout group) of one MMA are one core matrix apart (M = 128; 3 COUT rows used);
+//   X as planes [kx][cin group][row][column], three copies a column apart; then a plane of ones in
+//      channel 0, whose accumulator column for ky = 1 is the sum of dY: the bias gradient.
+// Rows and columns past those read whatever follows in shared memory and are never read back.
+// One CTA per SM, warp-specialised: four warps copy tiles into a ring of stages, one thread issues
+// the 8 MMAs of a tile (K = 16: two image rows).  The partial sums go to a scratch gradient
+// [tap][cout][cin] (bias after the weights) in 16-byte reductions, two lanes to a 32-byte sector;
+// unpack_grads_kernel lays it out as the parameters.
+// All nine taps in one MMA, because what bounds it is the operands' shared-memory reads: one MMA
+// per tap row, (kx, cin) x cout, reads A three times (2.2 times the time per tile), and one CTA per
+// SM, because every CTA ends with the whole gradient in reductions (5 us of a launch at two per SM).
+// 32 -> 32 on 16 x 128 x 128 pixels under ncu: 318 us with both operands transposed into K-major
+// tiles by 2-byte stores and scalar reductions at a 36-byte stride; 20 us now.
+constexpr int kWgTW = 8, kWgTH = 16;               // K = 128 pixels per tile
+constexpr int kWgStages = 4;
+constexpr int kWgThreads = 160;                    // four copying warps and the MMA warp
+template <int C> constexpr int wg_pad() { return 16 * (64 / C); }   // a pixel's groups in different banks
+template <int CIN> constexpr int wg_plane() { return kWgTH * kWgTW * 16 + wg_pad<CIN>(); }
+template <int COUT> constexpr int wg_core() { return kWgTW * 16 + wg_pad<COUT>(); }
 template <int CIN, int COUT>
-constexpr int wgrad_mtiles() { return (9 * CIN + 127) / 128; }
-
+constexpr int wgrad_stage_bytes() {
+  return (3 * (CIN / 8) + 1) * wg_plane<CIN>() + (kWgTH + 2) * (COUT / 8) * wg_core<COUT>();
+}
+// the last core matrices of the last stage's A operand end past its rows
 template <int CIN, int COUT>
-constexpr int wgrad_smem_bytes() {
-  return wgrad_mtiles<CIN, COUT>() * 16384 + (COUT / 8) * 1024 + (CIN / 8) * (kWgTile + 2) * (kWgTile + 2) * 16;
+constexpr int wgrad_smem_bytes() { return kWgStages * wgrad_stage_bytes<CIN, COUT>() + 16 * wg_core<COUT>(); }
+
+__device__ __forceinline__ void red_add4(float *p, float a, float b, float c, float d) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
+// Adds v[0..N), of this lane's row, to row[0..N) of every lane (rows of adjacent lanes exchange
+// quarters so that two lanes cover one 32-byte sector of one row per instruction).  Whole warps;
+// row may be null in adjacent pairs of lanes only.
+template <int N>
+__device__ __forceinline__ void red_add_rows(float *row, const float *v) {
+  const bool odd = threadIdx.x & 1;
+  const unsigned long long mine = reinterpret_cast<unsigned long long>(row);
+  float *const other = reinterpret_cast<float *>(__shfl_xor_sync(0xffffffffu, mine, 1));
+  float *const even_row = odd ? other : row, *const odd_row = odd ? row : other;
+#pragma unroll
+  for (int c = 0; c < N; c += 8) {
+    float r[4];   // even lanes: the odd row's first half sector; odd lanes: the even row's second
+#pragma unroll
+    for (int j = 0; j < 4; ++j) r[j] = __shfl_xor_sync(0xffffffffu, odd ? v[c + j] : v[c + 4 + j], 1);
+    if (row) {
+      if (odd) {
+        red_add4(even_row + c + 4, r[0], r[1], r[2], r[3]);
+        red_add4(odd_row + c + 4, v[c + 4], v[c + 5], v[c + 6], v[c + 7]);
+      } else {
+        red_add4(even_row + c, v[c], v[c + 1], v[c + 2], v[c + 3]);
+        red_add4(odd_row + c, r[0], r[1], r[2], r[3]);
+      }
+    }
+  }
 }
 
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(128)
-conv3x3_wgrad_tc_kernel(ConvDims d, const __nv_bfloat16 *__restrict__ X,
-                        const __nv_bfloat16 *__restrict__ dY, float *__restrict__ dW,
-                        float *__restrict__ db, int tiles_per_cta, uint32_t *__restrict__ status) {
-  constexpr int CG = CIN / 8, MT = wgrad_mtiles<CIN, COUT>(), HR = kWgTile + 2, HC = kWgTile + 2;
-  constexpr int ABYTES = MT * 16384, BBYTES = (COUT / 8) * 1024;
+__global__ void __launch_bounds__(kWgThreads, 1)
+conv3x3_wgrad_tc_kernel(ConvDims d, const __nv_bfloat16 *__restrict__ X, const __nv_bfloat16 *__restrict__ dY,
+                        float *__restrict__ dW, float *__restrict__ db, uint32_t *__restrict__ status) {
+  constexpr int CG = CIN / 8, OG = COUT / 8, XG = 3 * CG, HR = kWgTH + 2, S = kWgStages;
+  constexpr int XP = wg_plane<CIN>(), YC = wg_core<COUT>(), XROW = kWgTW * 16, YROW = OG * YC;
+  constexpr int STAGE = wgrad_stage_bytes<CIN, COUT>(), YOFF = (XG + 1) * XP;
+  constexpr int N = 3 * CIN + 16;   // the plane of ones and one of nothing: N is a multiple of 16
   extern __shared__ __align__(1024) uint8_t smem[];
-  uint8_t *as = smem, *bs = smem + ABYTES, *hs = smem + ABYTES + BBYTES;
   __shared__ uint32_t s_tmem;
-  __shared__ __align__(8) uint64_t s_bar;
+  __shared__ __align__(8) uint64_t s_full[S], s_empty[S], s_done;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int tx_n = (d.W + kWgTile - 1) / kWgTile, ty_n = (d.H + kWgTile - 1) / kWgTile;
+  const int tx_n = (d.W + kWgTW - 1) / kWgTW, ty_n = (d.H + kWgTH - 1) / kWgTH;
   const int n_tiles = d.B * tx_n * ty_n;
-  if (warp == 0) tc::tmem_alloc(&s_tmem, 128);
-  if (t == 0) tc::mbar_init(&s_bar, 1);
+  const int my_n = (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // grid <= n_tiles
+  for (int i = t; i < S * kWgTH * kWgTW; i += kWgThreads) {
+    const int stage = i / (kWgTH * kWgTW), q = i - stage * (kWgTH * kWgTW);
+    *reinterpret_cast<uint4 *>(smem + stage * STAGE + XG * XP + q * 16) = make_uint4(0x3f80u, 0u, 0u, 0u);
+  }
+  if (warp == 4) tc::tmem_alloc(&s_tmem, 128);
+  if (t == 0) {
+    for (int k = 0; k < S; ++k) {
+      tc::mbar_init(&s_full[k], 4);
+      tc::mbar_init(&s_empty[k], 1);
+    }
+    tc::mbar_init(&s_done, 1);
+  }
+  tc::fence_proxy_async();
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = s_tmem;
-  constexpr int BG = COUT / 8;           // 8-channel groups of dY
-  const int my_g = t % BG;               // every (pixel, group) entry of this thread has group my_g
-  float dbl[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  int issued = 0;
-  for (int q = 0; q < tiles_per_cta; ++q) {
-    const int tt = blockIdx.x * tiles_per_cta + q;
-    if (tt >= n_tiles) break;
-    const int b = tt / (tx_n * ty_n), rem = tt - b * (tx_n * ty_n);
-    const int y0 = (rem / tx_n) * kWgTile, x0 = (rem % tx_n) * kWgTile;
-    if (issued > 0) {   // the previous tile's MMAs still read A and B
-      if (!tc::mbar_wait(&s_bar, (issued - 1) & 1) && lane == 0) atomicOr(status, kStatusTimeout);
-      tc::fence_after_sync();
-    }
-    load_halo<CG>(hs, X, b, y0, x0, HR, HC, d.H, d.W);
-    // B[cout][pixel]: entry e = (pixel, group of 8 couts)
-    for (int e = t; e < 64 * BG; e += 128) {
-      const int p = e / BG, g = e - (e / BG) * BG;
-      const int y = y0 + p / kWgTile, x = x0 + (p % kWgTile);
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (y < d.H && x < d.W) v = __ldg(reinterpret_cast<const uint4 *>(dY + (((size_t)b * d.H + y) * d.W + x) * COUT) + g);
-      const __nv_bfloat16 *vb = reinterpret_cast<const __nv_bfloat16 *>(&v);
-      uint8_t *dst = bs + g * 1024 + (p >> 3) * 128 + (p & 7) * 2;
+  pdl_begin();
+  if (warp == 4) {
+    if (lane == 0) {
+      constexpr uint32_t idesc = tc::idesc_bf16_f32(128, N) | tc::kIdescMnMajorA | tc::kIdescMnMajorB;
+      for (int k = 0; k < my_n; ++k) {
+        const int st = k % S;
+        if (!tc::mbar_wait(&s_full[st], (k / S) & 1)) atomicOr(status, kStatusTimeout);
+        tc::fence_after_sync();
+        const uint32_t b0 = tc::smem_u32(smem + st * STAGE), a0 = b0 + YOFF;
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        *reinterpret_cast<__nv_bfloat16 *>(dst + c * 16) = vb[c];
-        dbl[c] += __bfloat162float(vb[c]);
+        for (int r = 0; r < kWgTH / 2; ++r)
+          tc::mma_bf16(tmem, tc::smem_desc(a0 + 2 * r * YROW, YROW, YC), tc::smem_desc(b0 + 2 * r * XROW, XROW, XP),
+                       idesc, k > 0 || r > 0);
+        tc::mma_commit(&s_empty[st]);
+      }
+      tc::mma_commit(&s_done);
+    }
+    __syncwarp();
+  } else {
+    // threads 0..95 copy X (24 CG of them one row of the three copies), threads 96..127 dY (8 OG a
+    // row): each thread one (shift, column, group) down the rows, so a copy costs a few additions
+    const bool mine_x = t < 96;
+    const int lt = mine_x ? t : t - 96;
+    const int lg = mine_x ? lt % CG : lt % OG, lc = (mine_x ? lt / CG : lt / OG) % kWgTW;
+    const int lkx = (lt / (CG * kWgTW)) % 3;                                             // X only
+    const int lrow = mine_x ? lt / (CG * kWgTW * 3) : lt / (OG * kWgTW), lstep = mine_x ? 4 / CG : 4 / OG;
+    const uint32_t ldst = mine_x ? (lkx * CG + lg) * XP + lrow * XROW + lc * 16
+                                 : YOFF + lrow * YROW + lg * YC + lc * 16;
+    for (int k = 0; k < my_n + 2; ++k) {
+      const int st = k % S;
+      if (k >= S && k < my_n && !tc::mbar_wait(&s_empty[st], (k / S - 1) & 1) && lane == 0)
+        atomicOr(status, kStatusTimeout);
+      if (k < my_n) {
+        const int tt = (int)blockIdx.x + k * (int)gridDim.x;
+        const int x0 = (tt % tx_n) * kWgTW, rest = tt / tx_n;
+        const int y0 = (rest % ty_n) * kWgTH, b = rest / ty_n;
+        uint32_t dst = tc::smem_u32(smem + st * STAGE) + ldst;
+        const ptrdiff_t img = (ptrdiff_t)b * d.H * d.W;
+        if (mine_x) {
+          const int x = x0 - 1 + lkx + lc;
+          const bool in_x = x >= 0 && x < d.W;
+          int y = y0 + lrow;
+          const __nv_bfloat16 *src = X + (img + (ptrdiff_t)y * d.W + x) * CIN + lg * 8;
+          const ptrdiff_t step = (ptrdiff_t)lstep * d.W * CIN;
+#pragma unroll 8
+          for (int row = lrow; row < kWgTH; row += lstep) {
+            const bool in = in_x && y < d.H;
+            // the three copies of a row read the same lines: through L1
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(in ? src : X),
+                         "r"(in ? 16 : 0)
+                         : "memory");
+            dst += lstep * XROW;
+            src += step;
+            y += lstep;
+          }
+        } else {
+          const int x = x0 + lc;
+          int y = y0 - 1 + lrow;
+          const __nv_bfloat16 *src = dY + (img + (ptrdiff_t)y * d.W + x) * COUT + lg * 8;
+          const ptrdiff_t step = (ptrdiff_t)lstep * d.W * COUT;
+#pragma unroll 6
+          for (int row = lrow; row < HR; row += lstep) {
+            const bool in = x < d.W && y >= 0 && y < d.H;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(in ? src : dY),
+                         "r"(in ? 16 : 0)
+                         : "memory");
+            dst += lstep * YROW;
+            src += step;
+            y += lstep;
+          }
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      if (k >= 2) {   // tile k - 2 has landed
+        asm volatile("cp.async.wait_group 2;" ::: "memory");
+        tc::fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&s_full[(k - 2) % S]);
       }
     }
-    __syncthreads();   // halo complete
-    // A[(tap, cin)][pixel]: entry e = (pixel, tap, channel group)
-    for (int e = t; e < 64 * 9 * CG; e += 128) {
-      const int cg = e % CG, pt = e / CG;
-      const int tap = pt % 9, p = pt / 9;
-      const int ky = tap / 3, kx = tap - 3 * ky;
-      const int oy = p / kWgTile, ox = p % kWgTile;
-      const uint4 v = *reinterpret_cast<const uint4 *>(hs + ((size_t)(cg * HR + oy + ky) * HC + ox + kx) * 16);
-      const __nv_bfloat16 *vb = reinterpret_cast<const __nv_bfloat16 *>(&v);
-      const int row = tap * CIN + cg * 8;    // 8 consecutive rows: one core matrix's rows
-      const int mt = row >> 7, i = row & 127;
-      uint8_t *dst = as + mt * 16384 + (i >> 3) * 1024 + (p >> 3) * 128 + (p & 7) * 2;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) *reinterpret_cast<__nv_bfloat16 *>(dst + c * 16) = vb[c];
-    }
-    tc::fence_proxy_async();
-    tc::fence_before_sync();
-    __syncthreads();
+    if (!tc::mbar_wait(&s_done, 0) && lane == 0) atomicOr(status, kStatusTimeout);
     tc::fence_after_sync();
-    if (t == 0) {
-      const uint32_t a0 = tc::smem_u32(as), b0 = tc::smem_u32(bs);
-      const uint32_t idesc = tc::idesc_bf16_f32(128, COUT);
-#pragma unroll
-      for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-        for (int kc = 0; kc < 4; ++kc)
-          tc::mma_bf16(tmem + mt * COUT, tc::smem_desc(a0 + mt * 16384 + kc * 256, 128, 1024),
-                       tc::smem_desc(b0 + kc * 256, 128, 1024), idesc, issued > 0 || kc > 0);
-      tc::mma_commit(&s_bar);
-    }
-    ++issued;
-  }
-  // bias gradient: lanes with the same channel group are BG apart within the warp
-#pragma unroll
-  for (int c = 0; c < 8; ++c)
-    for (int o = BG; o < 32; o <<= 1) dbl[c] += __shfl_xor_sync(0xffffffffu, dbl[c], o);
-  if (lane < BG)
-#pragma unroll
-    for (int c = 0; c < 8; ++c) atomicAdd(db + my_g * 8 + c, dbl[c]);
-  if (issued > 0) {
-    if (!tc::mbar_wait(&s_bar, (issued - 1) & 1) && lane == 0) atomicOr(status, kStatusTimeout);
-    tc::fence_after_sync();
+    // accumulator rows (2 - ky, cout), columns (kx, cin), then the ones
+    const int row = warp * 32 + lane, ky = 2 - row / COUT, co = row % COUT;
+    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
+    if (warp * 32 < 3 * COUT) {   // whole warps: 3 COUT is 96, or 48 with the rest skipped below
 #pragma unroll 1
-    for (int mt = 0; mt < MT; ++mt) {
-      float v[32];
-      const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + mt * COUT;
-      if (COUT == 32) tc::tmem_ld32(taddr, v);
-      else tc::tmem_ld16(taddr, v);
-      const int row = mt * 128 + warp * 32 + lane;
-      if (row < 9 * CIN) {
-        const int tap = row / CIN, ci = row - tap * CIN;
-#pragma unroll
-        for (int co = 0; co < COUT; ++co) atomicAdd(dW + ((size_t)co * CIN + ci) * 9 + tap, v[co]);
+      for (int kx = 0; kx < 3; ++kx) {
+        float v[32];
+        if (CIN == 32) tc::tmem_ld32(taddr + kx * CIN, v);
+        else tc::tmem_ld16(taddr + kx * CIN, v);
+        red_add_rows<CIN>(ky >= 0 ? dW + (size_t)((ky * 3 + kx) * COUT + co) * CIN : nullptr, v);
       }
+      float v[16];
+      tc::tmem_ld16(taddr + 3 * CIN, v);
+      if (ky == 1) atomicAdd(db + co, v[0]);
     }
+    tc::fence_before_sync();
   }
-  tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, 128);
+  tc::fence_after_sync();
+  if (warp == 4) tc::tmem_dealloc(tmem, 128);
 }
 
 // ------------------------------------------------------- CUDA-core helpers of the network
@@ -902,11 +979,6 @@ __global__ void pack_kernel(const float *__restrict__ w, int cin, int cout, int 
   }
 }
 
-// dW[cout][cin] += the centre tap of a 3x3 weight gradient g[cout][cin][9].
-__global__ void centre_tap_kernel(const float *__restrict__ g, int n, float *__restrict__ dW) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dW[i] += g[i * 9 + 4];
-}
-
 // Layer tables.  Residual network: ten 3x3 convolutions (16 -> 32, eight 32 -> 32, 32 -> 16).
 // Compact network: 3x3 16 -> 32, then the per-block layers 32 -> 32 and 32 -> 16.
 constexpr int kLayers = 10;   // the most layers of either network
@@ -927,6 +999,50 @@ size_t bias_offset(int arch, int l) {
 }
 size_t n_params(int arch) { return bias_offset(arch, n_layers(arch)); }
 
+// The scratch gradient of the weight-gradient kernels: per layer [9 taps][cout][cin], then [cout].
+size_t scratch_offset(int arch, int l) {
+  size_t o = 0;
+  for (int k = 0; k < l; ++k) o += ((size_t)9 * layer_in(arch, k) + 1) * layer_out(arch, k);
+  return o;
+}
+
+struct GradMap {   // per layer: parameters and scratch offsets
+  int n_layers, n_params;
+  int w[kLayers], b[kLayers], scratch[kLayers], cin[kLayers], cout[kLayers], taps[kLayers];
+};
+
+GradMap grad_map(int arch) {
+  GradMap m{};
+  m.n_layers = n_layers(arch);
+  m.n_params = (int)n_params(arch);
+  for (int l = 0; l < m.n_layers; ++l) {
+    m.w[l] = (int)weight_offset(arch, l);
+    m.b[l] = (int)bias_offset(arch, l);
+    m.scratch[l] = (int)scratch_offset(arch, l);
+    m.cin[l] = layer_in(arch, l);
+    m.cout[l] = layer_out(arch, l);
+    m.taps[l] = layer_taps(arch, l);
+  }
+  return m;
+}
+
+// The flat gradient, laid out as the parameters (W[cout][cin][taps] per layer, then the biases),
+// from the scratch gradient; a per-block layer takes the centre tap.
+__global__ void unpack_grads_kernel(GradMap m, const float *__restrict__ scratch, float *__restrict__ grads) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m.n_params; i += gridDim.x * blockDim.x) {
+    int l = m.n_layers - 1;
+    if (i < m.b[0]) {
+      while (i < m.w[l]) --l;
+      const int j = i - m.w[l], tap = m.taps[l] == 9 ? j % 9 : 4, rest = j / m.taps[l];
+      const int ci = rest % m.cin[l], co = rest / m.cin[l];
+      grads[i] = scratch[m.scratch[l] + (tap * m.cout[l] + co) * m.cin[l] + ci];
+    } else {
+      while (i < m.b[l]) --l;
+      grads[i] = scratch[m.scratch[l] + 9 * m.cin[l] * m.cout[l] + (i - m.b[l])];
+    }
+  }
+}
+
 int grid_1d(size_t n) {
   const size_t b = (n + 255) / 256;
   return (int)(b < 152 * 16 ? (b > 0 ? b : 1) : 152 * 16);
@@ -938,7 +1054,7 @@ int grid_1d(size_t n) {
 struct a3fr_cnn {
   int arch = A3FR_CNN_RESIDUAL;
   float *params = nullptr, *grads = nullptr, *adam_m = nullptr, *adam_v = nullptr;
-  float *wscratch = nullptr;   // a per-block layer's 3x3 weight gradient [32][32][9]
+  float *wscratch = nullptr;   // the gradients as the weight-gradient kernels leave them (scratch_offset)
   __nv_bfloat16 *wf[a3fr::kLayers] = {}, *wb[a3fr::kLayers] = {};
   size_t cap_px = 0;
   __nv_bfloat16 *x0 = nullptr, *h[5] = {}, *t[4] = {}, *g_r = nullptr, *gA = nullptr, *gB = nullptr, *gT = nullptr;
@@ -1031,9 +1147,10 @@ cudaError_t compact_fill(const ConvDims &d, const a3fr_cnn *n, uint32_t *status,
   return cudaGetLastError();
 }
 
+// Adds layer l's weight and bias gradients to the scratch gradient.
 template <int CIN, int COUT>
-cudaError_t wgrad(const ConvDims &d, const __nv_bfloat16 *X, const __nv_bfloat16 *dY, float *dW, float *db,
-                  uint32_t *status, cudaStream_t s) {
+cudaError_t wgrad(const a3fr_cnn *n, int l, const ConvDims &d, const __nv_bfloat16 *X, const __nv_bfloat16 *dY,
+                  cudaStream_t s) {
   constexpr int smem = wgrad_smem_bytes<CIN, COUT>();
   static bool attr[64] = {};
   int dev = 0;
@@ -1044,11 +1161,10 @@ cudaError_t wgrad(const ConvDims &d, const __nv_bfloat16 *X, const __nv_bfloat16
     if (e != cudaSuccess) return e;
     attr[dev] = true;
   }
-  const int tiles = d.B * ((d.H + kWgTile - 1) / kWgTile) * ((d.W + kWgTile - 1) / kWgTile);
-  const int ctas = tiles < 152 * 3 ? tiles : 152 * 3;
-  const int per = (tiles + ctas - 1) / ctas;
-  conv3x3_wgrad_tc_kernel<CIN, COUT><<<ctas, 128, smem, s>>>(d, X, dY, dW, db, per, status);
-  return cudaGetLastError();
+  const int tiles = d.B * ((d.H + kWgTH - 1) / kWgTH) * ((d.W + kWgTW - 1) / kWgTW);
+  float *dW = n->wscratch + scratch_offset(n->arch, l);
+  return launch_pdl(conv3x3_wgrad_tc_kernel<CIN, COUT>, tiles < 152 ? tiles : 152, kWgThreads, smem, s, d, X, dY, dW,
+                    dW + 9 * CIN * COUT, n->status);
 }
 
 #define CNN_CHECK(call)                                  \
@@ -1116,55 +1232,42 @@ int forward(a3fr_cnn *n, const float *img, const float *depth, int B, int H, int
   return A3FR_OK;
 }
 
-// Weight gradient of a per-block layer: the 3x3 kernel into the scratch, its centre tap added
-// to dW[cout][cin]; the bias gradient directly.
-template <int CIN, int COUT>
-int wgrad_1x1(a3fr_cnn *n, const ConvDims &d, const __nv_bfloat16 *X, const __nv_bfloat16 *dY, float *dW,
-              float *db, cudaStream_t s) {
-  CNN_CHECK(cudaMemsetAsync(n->wscratch, 0, sizeof(float) * CIN * COUT * 9, s));
-  CNN_CHECK((wgrad<CIN, COUT>(d, X, dY, n->wscratch, db, n->status, s)));
-  centre_tap_kernel<<<grid_1d((size_t)CIN * COUT), 256, 0, s>>>(n->wscratch, CIN * COUT, dW);
-  CNN_CHECK(cudaGetLastError());
-  return A3FR_OK;
-}
-
 // Gradients of the mean squared error of the prediction against target into n->grads.
 int backward(a3fr_cnn *n, const float *img, const float *target, int B, int H, int W, cudaStream_t s) {
   const ConvDims d{B, (H + 1) / 2, (W + 1) / 2};
   const size_t px = (size_t)d.B * d.H * d.W;
   const int A = n->arch;
-  float *G = n->grads;
-  CNN_CHECK(cudaMemsetAsync(G, 0, sizeof(float) * n_params(A), s));
+  CNN_CHECK(cudaMemsetAsync(n->wscratch, 0, sizeof(float) * scratch_offset(A, n_layers(A)), s));
   CNN_CHECK(cudaMemsetAsync(n->loss_acc, 0, sizeof(float), s));
   loss_kernel<<<grid_1d(px), 256, 0, s>>>(n->r, img, target, B, H, W, 1.0f / (3.0f * B * H * W), n->g_r,
                                           n->loss_acc);
   CNN_CHECK(cudaGetLastError());
   if (A == A3FR_CNN_COMPACT) {
     // r = W2 t + b2;  t = ReLU(W1 h + b1);  h = ReLU(conv0(x0) + b0)
-    int rc = wgrad_1x1<32, 16>(n, d, n->t[0], n->g_r, G + weight_offset(A, 2), G + bias_offset(A, 2), s);
-    if (rc != A3FR_OK) return rc;
+    CNN_CHECK((wgrad<32, 16>(n, 2, d, n->t[0], n->g_r, s)));
     CNN_CHECK((conv<16, 32>(d, n->g_r, n->wb[2], nullptr, nullptr, n->t[0], n->gA, kEpiMask, n->status, s)));
-    rc = wgrad_1x1<32, 32>(n, d, n->h[0], n->gA, G + weight_offset(A, 1), G + bias_offset(A, 1), s);
-    if (rc != A3FR_OK) return rc;
+    CNN_CHECK((wgrad<32, 32>(n, 1, d, n->h[0], n->gA, s)));
     CNN_CHECK((conv<32, 32>(d, n->gA, n->wb[1], nullptr, nullptr, n->h[0], n->gB, kEpiMask, n->status, s)));
-    CNN_CHECK((wgrad<16, 32>(d, n->x0, n->gB, G + weight_offset(A, 0), G + bias_offset(A, 0), n->status, s)));
-    return A3FR_OK;
+    CNN_CHECK((wgrad<16, 32>(n, 0, d, n->x0, n->gB, s)));
+  } else {
+    CNN_CHECK((wgrad<32, 16>(n, 9, d, n->h[4], n->g_r, s)));
+    CNN_CHECK((conv<16, 32>(d, n->g_r, n->wb[9], nullptr, nullptr, nullptr, n->gA, 0, n->status, s)));
+    __nv_bfloat16 *cur = n->gA, *nxt = n->gB;
+    for (int b = 3; b >= 0; --b) {
+      const int l2 = 2 + 2 * b, l1 = 1 + 2 * b;
+      CNN_CHECK((wgrad<32, 32>(n, l2, d, n->t[b], cur, s)));
+      CNN_CHECK((conv<32, 32>(d, cur, n->wb[l2], nullptr, nullptr, n->t[b], n->gT, kEpiMask, n->status, s)));
+      CNN_CHECK((wgrad<32, 32>(n, l1, d, n->h[b], n->gT, s)));
+      CNN_CHECK((conv<32, 32>(d, n->gT, n->wb[l1], nullptr, cur, b == 0 ? n->h[0] : nullptr, nxt,
+                              kEpiResid | (b == 0 ? kEpiMask : 0), n->status, s)));
+      __nv_bfloat16 *tmp = cur;
+      cur = nxt;
+      nxt = tmp;
+    }
+    CNN_CHECK((wgrad<16, 32>(n, 0, d, n->x0, cur, s)));
   }
-  CNN_CHECK((wgrad<32, 16>(d, n->h[4], n->g_r, G + weight_offset(A, 9), G + bias_offset(A, 9), n->status, s)));
-  CNN_CHECK((conv<16, 32>(d, n->g_r, n->wb[9], nullptr, nullptr, nullptr, n->gA, 0, n->status, s)));
-  __nv_bfloat16 *cur = n->gA, *nxt = n->gB;
-  for (int b = 3; b >= 0; --b) {
-    const int l2 = 2 + 2 * b, l1 = 1 + 2 * b;
-    CNN_CHECK((wgrad<32, 32>(d, n->t[b], cur, G + weight_offset(A, l2), G + bias_offset(A, l2), n->status, s)));
-    CNN_CHECK((conv<32, 32>(d, cur, n->wb[l2], nullptr, nullptr, n->t[b], n->gT, kEpiMask, n->status, s)));
-    CNN_CHECK((wgrad<32, 32>(d, n->h[b], n->gT, G + weight_offset(A, l1), G + bias_offset(A, l1), n->status, s)));
-    CNN_CHECK((conv<32, 32>(d, n->gT, n->wb[l1], nullptr, cur, b == 0 ? n->h[0] : nullptr, nxt,
-                            kEpiResid | (b == 0 ? kEpiMask : 0), n->status, s)));
-    __nv_bfloat16 *tmp = cur;
-    cur = nxt;
-    nxt = tmp;
-  }
-  CNN_CHECK((wgrad<16, 32>(d, n->x0, cur, G + weight_offset(A, 0), G + bias_offset(A, 0), n->status, s)));
+  unpack_grads_kernel<<<grid_1d(n_params(A)), 256, 0, s>>>(grad_map(A), n->wscratch, n->grads);
+  CNN_CHECK(cudaGetLastError());
   return A3FR_OK;
 }
 
@@ -1224,7 +1327,7 @@ int a3fr_cnn_create_arch(a3fr_cnn **out, int arch) {
             cudaMalloc(&n->grads, np * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&n->adam_m, np * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&n->adam_v, np * sizeof(float)) == cudaSuccess &&
-            cudaMalloc(&n->wscratch, 32 * 32 * 9 * sizeof(float)) == cudaSuccess &&
+            cudaMalloc(&n->wscratch, scratch_offset(arch, n_layers(arch)) * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&n->loss_acc, sizeof(float)) == cudaSuccess &&
             cudaMalloc(&n->status, sizeof(uint32_t)) == cudaSuccess;
   for (int l = 0; l < n_layers(arch) && ok; ++l) {   // 3x3 packs (a per-block layer: its centre tap)
