@@ -143,7 +143,7 @@ struct a3fr_scene {
   cudaStream_t capture_stream = nullptr;
   cudaGraphExec_t g_pre = nullptr, g_fov = nullptr, g_full = nullptr;
   uint64_t g_pre_key = 0, g_fov_key = 0, g_full_key = 0;
-  uint64_t g_pre_launches = 0;               // kernels in the precompute graph
+  uint64_t g_pre_launches = 0, g_fov_launches = 0, g_full_launches = 0;   // kernels in each graph
 
   int batch_mult = 1;                        // Gaussians staged per thread per composite batch
 
@@ -640,7 +640,7 @@ int enqueue_pre(a3fr_scene *s, int eyes, cudaStream_t stream, bool allow_resize,
   return A3FR_OK;
 }
 
-// The composite of a render (plan + composite, or composite alone for full resolution).
+// The composite of a render (plan + composite, then the interpolating fill).
 int enqueue_comp(a3fr_scene *s, const CompositeParams &cp, int uniform, uint8_t *cur, bool fill,
                  cudaStream_t stream, uint64_t *launches) {
   A3FR_CHECK(mark(s, A3FR_STAGE_COMPOSITE, stream));
@@ -756,9 +756,9 @@ int render(a3fr_scene *s, const a3fr_fovea *fv, float *out, cudaStream_t stream,
                          (uint64_t)eyes;
     cudaGraphExec_t *g = mode == Mode::kFull ? &s->g_full : &s->g_fov;
     uint64_t *gk = mode == Mode::kFull ? &s->g_full_key : &s->g_fov_key;
+    uint64_t *gl = mode == Mode::kFull ? &s->g_full_launches : &s->g_fov_launches;
     if (!*g || *gk != key) {
-      uint64_t k = 0;
-      rc = capture(s, g, &k, [&](cudaStream_t cs, uint64_t *l) {
+      rc = capture(s, g, gl, [&](cudaStream_t cs, uint64_t *l) {
         return enqueue_comp(s, hp.comp, 0, nullptr, fill, cs, l);
       });
       if (rc != A3FR_OK) return rc;
@@ -768,7 +768,7 @@ int render(a3fr_scene *s, const a3fr_fovea *fv, float *out, cudaStream_t stream,
       A3FR_CHECK(mark(s, k, stream));
     A3FR_CHECK(cudaGraphLaunch(*g, stream));
     A3FR_CHECK(mark(s, A3FR_N_STAGES, stream));
-    launches += (mode == Mode::kFull ? 1 : 2) + (fill ? 1 : 0);
+    launches += *gl;
   } else {
     rc = enqueue_comp(s, hp.comp, uniform, cur, fill, stream, &launches);
     if (rc != A3FR_OK) return rc;

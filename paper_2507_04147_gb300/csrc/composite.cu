@@ -28,8 +28,6 @@
 namespace a3fr {
 namespace {
 
-constexpr int kTile = 16;
-constexpr int kThreads = 256;          // 8 warps
 // Level of tile `tile` of eye `eye` (exactly rounded; the same decision as the definition).
 __device__ __forceinline__ int tile_level(const CompositeParams &p, int eye, int tile,
                                           const float *gaze) {
@@ -138,54 +136,21 @@ __device__ __forceinline__ void tile_interval(const CompositeParams &p, int gt, 
   *hi_out = hi;
 }
 
-// Work plan of one 16-pixel-tile composite launch: entries (tile << 2 | lo) bucketed by
-// hi - lo in plan[(hi - lo - 1) * n_ranges + slot], the bucket sizes in plan_counts[0..3].
-__global__ void __launch_bounds__(256)
-plan_kernel(const CompositeParams *__restrict__ pp, const float *__restrict__ gaze_ring,
-            const RoundPlan *__restrict__ round, int uniform, uint8_t *__restrict__ cur,
-            uint8_t *__restrict__ levels, uint32_t *__restrict__ plan,
-            uint32_t *__restrict__ plan_counts, const uint2 *__restrict__ ranges,
-            const uint32_t *__restrict__ thresholds) {
-  pdl_begin();
-  const CompositeParams &p = *pp;
-  const float *gaze = gaze_ring + 4 * p.gaze_slot;
-  const int n_ranges = p.n_eyes * p.n_tiles;
-  const int gt = blockIdx.x * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  int lo = 0, count = 0;
-  if (gt < n_ranges) {
-    int hi;
-    tile_interval(p, gt, gaze, round, uniform, cur, levels, ranges, thresholds, &lo, &hi);
-    count = hi > lo ? hi - lo : 0;
-  }
-  for (int c = 1; c <= 4; ++c) {
-    const unsigned m = __ballot_sync(0xffffffffu, count == c);
-    if (!m) continue;
-    const int leader = __ffs(m) - 1;
-    uint32_t base = 0;
-    if (lane == leader) base = atomicAdd(plan_counts + (c - 1), (uint32_t)__popc(m));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (count == c)
-      plan[(size_t)(c - 1) * n_ranges + base + __popc(m & ((1u << lane) - 1u))] =
-          ((uint32_t)gt << 2) | (uint32_t)lo;
-  }
-}
-
-// Work plan of one 32-pixel-tile composite launch (composite_px_kernel).  A tile rendering
-// the P = hi - lo labels (lo, hi] is two work items, its top and bottom halves; a tile with
-// no instances is one item that only writes background.  Items go into kItemClasses classes by the tile's
-// instance count (class 0: none; class c: 4^(c-1) <= count < 4^c; the last class unbounded)
-// and the composite takes the heaviest class first, so the longest items start first and
-// the short ones fill in behind them.  items[c * 4 * n_ranges + slot] = gt << 6 |
-// (P - 1) << 4 | region << 2 | lo, class sizes in class_counts[0..kItemClasses).
+// Work plan of one composite launch (composite_px_kernel).  A tile rendering the P = hi - lo
+// labels (lo, hi] is `parts` work items (halves of the tile, or the whole of it); a tile with no
+// instances is one item that only writes background.  Items go into kItemClasses classes by the
+// tile's instance count (class 0: none; class c: 4^(c-1) <= count < 4^c; the last class unbounded)
+// and the composite takes the heaviest class first, so the longest items start first and the
+// short ones fill in behind them.  items[c * 4 * n_ranges + slot] = gt << 6 | (P - 1) << 4 |
+// region << 2 | lo, class sizes in class_counts[0..kItemClasses).
 constexpr int kItemClasses = 8;
 
 __global__ void __launch_bounds__(256)
-plan32_kernel(const CompositeParams *__restrict__ pp, const float *__restrict__ gaze_ring,
-              const RoundPlan *__restrict__ round, int uniform, uint8_t *__restrict__ cur,
-              uint8_t *__restrict__ levels, uint32_t *__restrict__ items,
-              uint32_t *__restrict__ class_counts, const uint2 *__restrict__ ranges,
-              const uint32_t *__restrict__ thresholds) {
+plan_kernel(const CompositeParams *__restrict__ pp, const float *__restrict__ gaze_ring,
+            const RoundPlan *__restrict__ round, int uniform, int parts, uint8_t *__restrict__ cur,
+            uint8_t *__restrict__ levels, uint32_t *__restrict__ items,
+            uint32_t *__restrict__ class_counts, const uint2 *__restrict__ ranges,
+            const uint32_t *__restrict__ thresholds) {
   pdl_begin();
   const CompositeParams &p = *pp;
   const float *gaze = gaze_ring + 4 * p.gaze_slot;
@@ -198,7 +163,7 @@ plan32_kernel(const CompositeParams *__restrict__ pp, const float *__restrict__ 
   const int P = hi - lo;
   const uint2 r = ranges[gt];
   const uint32_t count = r.y > r.x ? r.y - r.x : 0u;
-  const int n_items = count == 0u ? 1 : 2;
+  const int n_items = count == 0u ? 1 : parts;
   const int cls = count == 0u ? 0 : min(kItemClasses - 1, 1 + (31 - __clz(count)) / 2);
   const uint32_t slot = atomicAdd(class_counts + cls, (uint32_t)n_items);
   uint32_t *dst = items + (size_t)cls * 4 * n_ranges + slot;
@@ -247,286 +212,35 @@ __device__ __forceinline__ bool falloff_reaches(float A, float B, float C, float
   return best >= thr;
 }
 
-// Barrier of a staging group of `size` threads (64, 128 or 256) with barrier id `bar`
-// (1..4).  The ids are literals so the kernel reserves 5 hardware barriers, not 16 (the
-// per-SM barrier budget would otherwise cap residency at 4 CTAs).
-__device__ __forceinline__ void group_sync(int size, int bar) {
-  switch (bar) {
-    case 1: asm volatile("bar.sync 1, %0;" ::"r"(size) : "memory"); break;
-    case 2: asm volatile("bar.sync 2, %0;" ::"r"(size) : "memory"); break;
-    case 3: asm volatile("bar.sync 3, %0;" ::"r"(size) : "memory"); break;
-    default: asm volatile("bar.sync 4, %0;" ::"r"(size) : "memory"); break;
-  }
-}
-
-template <bool kAux, bool kFull, int kMult>
-__global__ void __launch_bounds__(kThreads, 6)
-composite_kernel(const CompositeParams *__restrict__ pp, const float *__restrict__ rec, int n,
-                 const uint2 *__restrict__ ranges, const uint32_t *__restrict__ kept,
-                 const uint32_t *__restrict__ vals, const uint32_t *__restrict__ plan,
-                 const uint32_t *__restrict__ plan_counts, int incremental,
-                 uint8_t *__restrict__ levels, float *__restrict__ t_final,
-                 uint32_t *__restrict__ n_contrib, float *__restrict__ depth,
-                 unsigned long long *__restrict__ counters) {
-  pdl_begin();
-  const CompositeParams &p = *pp;   // per-render parameters in device memory
-  float *out = p.out;
-  __shared__ float4 s_geo[kThreads * kMult];   // u, v, -0.5 log2e a, -log2e b
-  __shared__ float2 s_cz[kThreads * kMult];    // -0.5 log2e c, camera-space depth
-  __shared__ float4 s_rgb[kThreads * kMult];   // r, g, b, opacity
-  __shared__ int s_done[kThreads / 32];
-  __shared__ float s_out[4][kTile][kTile * 3];   // the tiles of the CTA, assembled for stores
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_ranges = p.n_eyes * p.n_tiles;
-
-  // ---- which tile, which labels (lo, level], which staging group; a label group is
-  // two warps, and group = the label index (0 = top-left) this warp pair renders
-  int gtile = -1, group = warp >> 1, level = 4, lo = 0, gsize = kThreads, gbar = 1, gfirst = 0;
-  if (kFull) {
-    gtile = blockIdx.x;
-    if (threadIdx.x == 0) levels[gtile] = 4;
-  } else {
-    const int c = blockIdx.x;
-    const int n4 = plan_counts[3], n3 = plan_counts[2], n2 = plan_counts[1], n1 = plan_counts[0];
-    const int c3 = n4 + n3, c2 = c3 + (n2 + 1) / 2, c1 = c2 + (n1 + 3) / 4;
-    uint32_t entry = 0xffffffffu;
-    int count = 4;
-    if (c < n4) {
-      entry = plan[3 * (size_t)n_ranges + c];
-    } else if (c < c3) {
-      entry = plan[2 * (size_t)n_ranges + (c - n4)];
-      count = 3;
-    } else if (c < c2) {
-      const int half = warp >> 2;
-      const int slot = 2 * (c - c3) + half;
-      count = 2;
-      group = (warp >> 1) & 1;
-      gsize = 128;
-      gbar = 1 + half;
-      gfirst = half * 128;
-      if (slot < n2) entry = plan[(size_t)n_ranges + slot];
-    } else if (c < c1) {
-      const int quarter = warp >> 1;
-      const int slot = 4 * (c - c2) + quarter;
-      count = 1;
-      group = 0;
-      gsize = 64;
-      gbar = 1 + quarter;
-      gfirst = quarter * 64;
-      if (slot < n1) entry = plan[slot];
-    } else {
-      return;
-    }
-    if (entry == 0xffffffffu) return;   // a partly filled pair or quad: these warps have no tile
-    gtile = (int)(entry >> 2);
-    lo = (int)(entry & 3u);
-    level = lo + count;
-    group += lo;
-  }
-  const int eye = gtile / p.n_tiles;
-  const int tile = gtile - eye * p.n_tiles;
-  const int tx = tile % p.tiles_x, ty = tile / p.tiles_x;
-
-  // ---- this lane's pixel: label `group` of block (bx, by) of the tile's 8x8 blocks
-  const int ox = (group == 1 || group == 2) ? 1 : 0;   // BR, TR
-  const int oy = (group == 1 || group == 3) ? 1 : 0;   // BR, BL
-  const int bx = lane & 7, by = (warp & 1) * 4 + (lane >> 3);
-  const int px = tx * kTile + 2 * bx + ox, py = ty * kTile + 2 * by + oy;
-  const bool inside = group >= lo && group < level && px < p.width && py < p.height;
-  const float fpx = (float)px, fpy = (float)py;
-
-  uint2 range = ranges[gtile];
-  const uint32_t n_kept = *kept;   // fewer than the instances only after a capacity overflow
-  range.x = min(range.x, n_kept);
-  range.y = min(range.y, n_kept);
-  const float *rec_eye = rec + (size_t)eye * n * kRec;
-
-  float T = 1.0f, C0 = 0.0f, C1 = 0.0f, C2 = 0.0f;
-  float Z = 0.0f;                      // expected depth (auxiliary output)
-  uint32_t last = 0;                   // 1-based position of the last contributor
-  uint32_t stop = 0;                   // Gaussians evaluated when the pixel stopped
-  uint32_t blended = 0;                // Gaussians blended into the pixel (auxiliary mode)
-  bool done = !inside;
-  uint32_t staged = 0;
-  if (kFull) {   // compile-time layout: one level-4 tile, the whole CTA stages together
-    group = warp >> 1;
-    level = 4;
-    lo = 0;
-    gsize = kThreads;
-    gbar = 1;
-    gfirst = 0;
-  }
-  const int gt = threadIdx.x - gfirst;   // thread index inside the staging group
-  const int sbase = gfirst * kMult;      // the group's staging slots
-  const uint32_t bsz = (uint32_t)(gsize * kMult);   // Gaussians per batch
-
-  for (uint32_t start = range.x; start < range.y; start += bsz) {
-    // stop when every pixel of the staging group is done
-    const bool wdone = __all_sync(0xffffffffu, done);
-    if (lane == 0) s_done[warp] = wdone;
-    group_sync(gsize, gbar);
-    bool all = true;
-    for (int w = gfirst >> 5; w < (gfirst + gsize) >> 5; ++w) all = all && s_done[w];
-    if (all) break;
-    const uint32_t cnt = min(bsz, range.y - start);
-    staged += cnt;
-#pragma unroll
-    for (int j = 0; j < kMult; ++j) {
-      const uint32_t slot = (uint32_t)(gt + j * gsize);
-      if (slot < cnt) {
-        const uint32_t gidx = min(vals[start + slot], (uint32_t)(n - 1));   // in range unless a sort failed
-        const float4 *r4 = reinterpret_cast<const float4 *>(rec_eye + (size_t)gidx * kRec);
-        const float4 a = __ldg(r4), b = __ldg(r4 + 1), c = __ldg(r4 + 2);
-        s_geo[sbase + slot] = make_float4(a.x, a.y, __fmul_rn(-0.5f * kLog2e, a.z), __fmul_rn(-kLog2e, a.w));
-        s_cz[sbase + slot] = make_float2(__fmul_rn(-0.5f * kLog2e, b.x), c.y);
-        s_rgb[sbase + slot] = make_float4(b.z, b.w, c.x, b.y);
-      } else if (slot < ((cnt + 3u) & ~3u)) {
-        // padding up to a multiple of 4: zero opacity never passes the 1/255 test
-        s_geo[sbase + slot] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        s_cz[sbase + slot] = make_float2(0.0f, 0.0f);
-        s_rgb[sbase + slot] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      }
-    }
-    group_sync(gsize, gbar);
-    if (!__all_sync(0xffffffffu, done)) {
-      // Branch-free blending: every lane evaluates every Gaussian of the batch and the
-      // update is predicated (a lane that is done, or outside the Gaussian's support or
-      // below 1/255, keeps its state), so the warp never splits on the accept test.
-      const uint32_t cnt4 = (cnt + 3u) & ~3u;
-      const uint32_t pos0 = start - range.x + 1;
-      for (uint32_t k = 0; k < cnt4; k += 4) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int e = sbase + (int)k + j;
-          const float4 geo = s_geo[e];
-          const float2 cz = s_cz[e];
-          const float cc = cz.x;
-          const float4 rgb = s_rgb[e];
-          const float dx = __fsub_rn(geo.x, fpx), dy = __fsub_rn(geo.y, fpy);
-          // power * log2(e) = -0.5 log2e (a dx^2 + c dy^2) - log2e b dx dy
-          const float pw = falloff_log2(geo.z, geo.w, cc, dx, dy);
-          const float alpha = blend_alpha(rgb.w, pw);
-          const float tt = __fmul_rn(T, __fsub_rn(1.0f, alpha));
-          const bool ok = !done && pw <= 0.0f && alpha >= 1.0f / 255.0f;
-          const bool fin = ok && tt < 0.0001f;    // this Gaussian would end the pixel: stop
-          const bool upd = ok && !fin;
-          const uint32_t pos = pos0 + k + (uint32_t)j;
-          const float w = upd ? alpha * T : 0.0f;
-          C0 += rgb.x * w;
-          C1 += rgb.y * w;
-          C2 += rgb.z * w;
-          if (kAux) {
-            Z += cz.y * w;
-            blended += upd ? 1u : 0u;
-          }
-          T = upd ? tt : T;
-          last = upd ? pos : last;
-          stop = fin ? pos : stop;
-          done = done || fin;
-        }
-        if (__all_sync(0xffffffffu, done)) break;
-      }
-    }
-    group_sync(gsize, gbar);   // the next batch overwrites the staged Gaussians
-  }
-  if (inside && !done) stop = range.y - range.x;
-
-  // ---- outputs.  A tile rendered from label 0 is assembled in shared memory (its pixel,
-  // and for label 1 the inherited pixels of its block) and stored row by row; a later
-  // round (lo > 0) stores only the pixels it rendered, keeping the others.
-  if (!kFull && incremental) {
-    if (inside) {
-      float *o = out + (((size_t)eye * p.height + py) * p.width + px) * 3;
-      o[0] = C0;
-      o[1] = C1;
-      o[2] = C2;
-      if (kAux) {
-        const size_t pix = ((size_t)eye * p.height + py) * p.width + px;
-        t_final[pix] = T;
-        n_contrib[pix] = last;
-        depth[pix] = Z;
-      }
-    }
-  } else {
-    const int slot = gfirst >> 6 >> (gsize == 256 ? 2 : (gsize == 128 ? 1 : 0));   // tile slot
-    const int lx = 2 * bx + ox, ly = 2 * by + oy;
-    if (inside) {
-      float *o = &s_out[slot][ly][3 * lx];
-      o[0] = C0;
-      o[1] = C1;
-      o[2] = C2;
-      if (kAux) {
-        const size_t pix = ((size_t)eye * p.height + py) * p.width + px;
-        t_final[pix] = T;
-        n_contrib[pix] = last;
-        depth[pix] = Z;
-      }
-      if (group == 0) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          // inherited pixels of the block: BR (label 2), TR (label 3), BL (label 4)
-          const int dx = k < 2 ? 1 : 0, dy = k == 1 ? 0 : 1;
-          if (level < k + 2 && px + dx < p.width && py + dy < p.height) {
-            float *f = &s_out[slot][ly + dy][3 * (lx + dx)];
-            f[0] = C0;
-            f[1] = C1;
-            f[2] = C2;
-            if (kAux) {
-              const size_t pix = ((size_t)eye * p.height + py + dy) * p.width + px + dx;
-              t_final[pix] = T;
-              n_contrib[pix] = last;
-        depth[pix] = Z;
-            }
-          }
-        }
-      }
-    }
-    group_sync(gsize, gbar);
-    const int w_tile = min(kTile, p.width - tx * kTile);
-    const int h_tile = min(kTile, p.height - ty * kTile);
-    const size_t row = (size_t)p.width * 3;
-    float *dst = out + ((size_t)eye * p.height + ty * kTile) * row + (size_t)tx * kTile * 3;
-    for (int f = gt; f < kTile * kTile * 3; f += gsize) {
-      const int r = f / (3 * kTile), c = f - r * (3 * kTile);
-      if (r < h_tile && c < 3 * w_tile) dst[(size_t)r * row + c] = s_out[slot][r][c];
-    }
-  }
-
-  // ---- statistics: evaluations of this warp, records staged by this staging group, and
-  // (auxiliary mode) blends
-  unsigned long long ev = stop, bl = blended;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    ev += __shfl_xor_sync(0xffffffffu, ev, o);
-    if (kAux) bl += __shfl_xor_sync(0xffffffffu, bl, o);
-  }
-  if (lane == 0) {
-    if (kAux && ev) atomicAdd(counters, ev);
-    if (gt == 0 && staged) atomicAdd(counters + 1, (unsigned long long)staged);
-    if (kAux && bl) atomicAdd(counters + 2, bl);
-  }
-}
-
-
-// 32 x 32 tiles (the paper's tiling, Sec. 3.5): a tile is 16 x 16 blocks of 2 x 2 pixels and
-// a tile of labels (lo, hi] renders those P = hi - lo labels of every block and no others (the
-// paper's groups above the level exit; here their pixels are never assigned).  Work items are
-// half tiles (16 x 8 blocks): one persistent launch renders every item of the plan
-// (plan32_kernel) -- both eyes, every layer -- taking items heaviest class first from an
-// atomic counter, so the longest lists start first and the short ones fill in behind them,
-// and a heavy tile is rendered by two CTAs at once.  A 128-thread CTA renders one item: each
-// lane the P pixels of one block, so a staged Gaussian is set up once for the lane's P
-// pixels; each warp covers 8 x 4 blocks (a 16 x 8 pixel area).  Per batch the CTA stages the
-// tile's next Gaussians in shared memory with the box where each can reach alpha = 1/255;
-// every warp builds its hit list (box test, then the exact falloff over its patch: a
-// Gaussian left out has alpha < 1/255 at every pixel of the patch, so no output bit changes)
-// and blends only those, front to back, with the 1/255 skip, the 0.99 clamp and the 1e-4
-// stop.  The per-pixel arithmetic is the same as everywhere else, so images do not depend on
-// how tiles are cut into items.  A tile rendered from label 0 also writes its inherited
-// pixels (the labels above hi take the top-left value).
+// A tile of labels (lo, hi] renders those P = hi - lo labels of every 2 x 2 block and no others (the
+// paper's groups above the level exit; here their pixels are never assigned).  One persistent
+// launch renders every item of the plan (plan_kernel) -- both eyes, every layer -- taking items
+// heaviest class first from an atomic counter, so the longest lists start first and the short
+// ones fill in behind them.  A 128-thread CTA renders one item.  Per batch it stages the tile's
+// next Gaussians in shared memory with the box where each can reach alpha = 1/255; every warp
+// builds the hit list of its patch (box test, then the exact falloff over the patch: a Gaussian
+// left out has alpha < 1/255 at every pixel of the patch, so no output bit changes) and blends
+// only those, front to back, with the 1/255 skip, the 0.99 clamp and the 1e-4 stop.  The per-pixel
+// arithmetic is the same in every shape, so images do not depend on how tiles are cut into items.
+// A tile rendered from label 0 also writes its inherited pixels (the labels above hi take the
+// top-left value).  Three shapes:
+//   kTile32       32-pixel tiles (the paper's, Sec. 3.5): an item is half a tile, a lane the P
+//                 pixels of one block, so a staged Gaussian is set up once for them; a warp's
+//                 patch is 16 x 8 pixels.
+//   kTile16       16-pixel tiles: an item is a tile, a warp's patch 8 x 8 pixels, two pixels a lane.
+//                 Bound by issue, as kTile32; every warp walking the whole list of its tile, one
+//                 pixel a lane, took 254 us on the 1M-Gaussian 1920 x 1080 full render (ncu), this
+//                 shape 117 us.
+//   kTile16Split  the same in half tiles, a patch 8 x 4 pixels, one pixel a lane: for renders with
+//                 too few tiles to fill the device, which are bound by the longest list's chain of
+//                 blends; fewer Gaussians reach the smaller patch.
+enum : int { kTile32 = 0, kTile16 = 1, kTile16Split = 2 };
 constexpr int kHalfThreads = 128;
 constexpr int kBatch = 256;   // Gaussians staged per batch (times the staging multiple)
+// 16-pixel tiles are split in halves up to this many tiles per SM (of about 9 CTAs resident).  Whole
+// render, split / not: 256 tiles 163 / 188 us, 825 tiles (training step) 420 / 451 us, 4,096 tiles
+// (training step) 896 / 889 us, 5,670 tiles 241 / 227 us, 8,160 tiles 616 / 567 us.
+constexpr int kSplitTilesPerSm = 16;
 
 __device__ __forceinline__ int label_dx(int L) { return (L == 1 || L == 2) ? 1 : 0; }
 __device__ __forceinline__ int label_dy(int L) { return (L == 1 || L == 3) ? 1 : 0; }
@@ -566,7 +280,7 @@ __device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
 }
 
 template <int kMult>
-struct HalfSmem {
+struct ItemSmem {
   float4 geo[kBatch * kMult];
   float2 cz[kBatch * kMult];
   float4 rgb[kBatch * kMult];
@@ -578,48 +292,36 @@ struct HalfSmem {
   uint32_t item;
 };
 
-// One item: labels lo .. lo + P - 1 of the blocks of half `half` of tile gtile (kLo0: lo is
-// 0, so the lane's pixel offsets are known at compile time).  Without the auxiliary outputs
-// a finished pixel is marked by T = 0 (a live pixel keeps T >= 1e-4): skipped Gaussians then
-// blend with alpha 0, which leaves T and the colour bit for bit as they were, and every
-// later Gaussian of a finished pixel stops with weight 0.  With them the loop also keeps the
-// final transmittance, the last contributor and the evaluation and blend counts.
-template <int P, bool kAux, int kMult, bool kLo0>
-__device__ __forceinline__ void render_half(HalfSmem<kMult> &sm, const CompositeParams &p, const float *rec,
-                                            int n, uint2 range, int gtile, int half, int lo,
-                                            bool inherit, const uint32_t *vals, float *t_final,
-                                            uint32_t *n_contrib, float *depth,
-                                            unsigned long long &ev, unsigned long long &bl,
-                                            unsigned long long &staged) {
-  constexpr int T32 = 32;
+// The pixels of one lane: P pixel centres (in pairs), which of them are to be rendered, and the
+// warp's patch -- the span of the pixel centres of all its lanes.
+template <int P>
+struct LanePixels {
+  float x[P], y[P];
+  bool inside[P];
+  float wx0, wx1, wy0, wy1;
+};
+
+// One item, by the whole CTA: the Gaussians of a tile's list blended into every lane's pixels.
+// Without the auxiliary outputs a finished pixel is marked by T = 0 (a live pixel keeps
+// T >= 1e-4): skipped Gaussians then blend with alpha 0, which leaves T and the colour bit for
+// bit as they were, and every later Gaussian of a finished pixel stops with weight 0.  With them
+// the loop also keeps the final transmittance, the last contributor and the evaluation and blend
+// counts.  inherit: pixel 0 is the top-left one of the block at (px0, py0), and the labels from
+// hi on take its value.
+template <int P, bool kAux, int kMult>
+__device__ __forceinline__ void render_pixels(ItemSmem<kMult> &sm, const CompositeParams &p, const float *rec,
+                                              int n, int eye, uint2 range, const LanePixels<P> &lp,
+                                              bool inherit, int hi, int px0, int py0,
+                                              const uint32_t *vals,
+                                              float *t_final, uint32_t *n_contrib, float *depth,
+                                              unsigned long long &ev, unsigned long long &bl,
+                                              unsigned long long &staged) {
   constexpr int NB = kBatch * kMult;
   float *out = p.out;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int hi = lo + P;
-  const int eye = gtile / p.n_tiles;
-  const int tile = gtile - eye * p.n_tiles;
-  const int tx = tile % p.tiles_x, ty = tile / p.tiles_x;
-  const int bx = (lane & 7) + 8 * (warp & 1), by = 8 * half + 4 * (warp >> 1) + (lane >> 3);
-  const int px0 = tx * T32 + 2 * bx, py0 = ty * T32 + 2 * by;   // the block's top-left pixel
-  float fpx[P], fpy[P];
-  bool inside[P];
-  int any_ox = 0, all_ox = 1, any_oy = 0, all_oy = 1;
-#pragma unroll
-  for (int k = 0; k < P; ++k) {
-    const int L = kLo0 ? k : lo + k;
-    const int ox = label_dx(L), oy = label_dy(L);
-    any_ox |= ox;
-    all_ox &= ox;
-    any_oy |= oy;
-    all_oy &= oy;
-    inside[k] = px0 + ox < p.width && py0 + oy < p.height;
-    fpx[k] = (float)(px0 + ox);
-    fpy[k] = (float)(py0 + oy);
-  }
-  // the warp's patch: the span of its pixels (one label: every other pixel of 16 x 8)
-  const int wxb = tx * T32 + 16 * (warp & 1), wyb = ty * T32 + 16 * half + 8 * (warp >> 1);
-  const float wx0 = (float)(wxb + all_ox), wx1 = (float)(wxb + 14 + any_ox);
-  const float wy0 = (float)(wyb + all_oy), wy1 = (float)(wyb + 6 + any_oy);
+  const float (&fpx)[P] = lp.x, (&fpy)[P] = lp.y;
+  const bool (&inside)[P] = lp.inside;
+  const float wx0 = lp.wx0, wx1 = lp.wx1, wy0 = lp.wy0, wy1 = lp.wy1;
   const float *rec_eye = rec + (size_t)eye * n * kRec;
 
   float T[P], C0[P], C1[P], C2[P], Z[P];
@@ -845,7 +547,6 @@ __device__ __forceinline__ void render_half(HalfSmem<kMult> &sm, const Composite
     }
   }
   if (inherit && inside[0]) {
-    // the inherited pixels of the block: the labels above the level take the top-left value
     for (int L = hi; L < 4; ++L) {
       const int x = px0 + label_dx(L), y = py0 + label_dy(L);
       if (x >= p.width || y >= p.height) continue;
@@ -862,8 +563,76 @@ __device__ __forceinline__ void render_half(HalfSmem<kMult> &sm, const Composite
   }
 }
 
-template <bool kAux, int kMult>
-__global__ void __launch_bounds__(kHalfThreads, kAux ? 6 : 7)
+// 32-pixel tiles: labels lo .. lo + P - 1 of the 16 x 8 blocks of half `half` of the tile, a lane
+// the P pixels of one block, a warp 8 x 4 blocks (kLo0: lo is 0, so the lane's pixel offsets are
+// known at compile time).
+template <int P, bool kLo0>
+__device__ __forceinline__ LanePixels<P> pixels32(const CompositeParams &p, int tx, int ty, int half, int lo,
+                                                  int &px0, int &py0) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int bx = (lane & 7) + 8 * (warp & 1), by = 8 * half + 4 * (warp >> 1) + (lane >> 3);
+  px0 = tx * 32 + 2 * bx;
+  py0 = ty * 32 + 2 * by;   // the block's top-left pixel
+  LanePixels<P> lp;
+  int any_ox = 0, all_ox = 1, any_oy = 0, all_oy = 1;
+#pragma unroll
+  for (int k = 0; k < P; ++k) {
+    const int L = kLo0 ? k : lo + k;
+    const int ox = label_dx(L), oy = label_dy(L);
+    any_ox |= ox;
+    all_ox &= ox;
+    any_oy |= oy;
+    all_oy &= oy;
+    lp.inside[k] = px0 + ox < p.width && py0 + oy < p.height;
+    lp.x[k] = (float)(px0 + ox);
+    lp.y[k] = (float)(py0 + oy);
+  }
+  // the warp's patch: the span of its pixels (one label: every other pixel of 16 x 8)
+  const int wxb = tx * 32 + 16 * (warp & 1), wyb = ty * 32 + 16 * half + 8 * (warp >> 1);
+  lp.wx0 = (float)(wxb + all_ox);
+  lp.wx1 = (float)(wxb + 14 + any_ox);
+  lp.wy0 = (float)(wyb + all_oy);
+  lp.wy1 = (float)(wyb + 6 + any_oy);
+  return lp;
+}
+
+// 16-pixel tiles: labels lo .. lo + P - 1 of a warp's patch of 4 x BH blocks (BH 4: the CTA's four
+// warps cover the tile; BH 2: half `half` of it).  The lanes are the patch's blocks times 8 / BH
+// label slots; a slot is Q consecutive labels (Q 2 with BH 4 when P > 2, else 1).
+template <int Q, int BH>
+__device__ __forceinline__ LanePixels<Q> pixels16(const CompositeParams &p, int tx, int ty, int half, int lo, int P,
+                                                  int &px0, int &py0) {
+  constexpr int NB = 4 * BH;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int wxb = tx * 16 + 8 * (warp & 1), wyb = ty * 16 + (BH == 4 ? 0 : 8 * half) + 2 * BH * (warp >> 1);
+  const int blk = lane % NB, slot = lane / NB;
+  px0 = wxb + 2 * (blk & 3);
+  py0 = wyb + 2 * (blk >> 2);
+  LanePixels<Q> lp;
+#pragma unroll
+  for (int k = 0; k < Q; ++k) {
+    const int L = lo + slot * Q + k;
+    const int x = px0 + label_dx(L), y = py0 + label_dy(L);
+    lp.inside[k] = slot * Q + k < P && x < p.width && y < p.height;
+    lp.x[k] = (float)x;
+    lp.y[k] = (float)y;
+  }
+  int any_ox = 0, all_ox = 1, any_oy = 0, all_oy = 1;
+  for (int L = lo; L < lo + P; ++L) {
+    any_ox |= label_dx(L);
+    all_ox &= label_dx(L);
+    any_oy |= label_dy(L);
+    all_oy &= label_dy(L);
+  }
+  lp.wx0 = (float)(wxb + all_ox);
+  lp.wx1 = (float)(wxb + 6 + any_ox);
+  lp.wy0 = (float)(wyb + all_oy);
+  lp.wy1 = (float)(wyb + 2 * (BH - 1) + any_oy);
+  return lp;
+}
+
+template <bool kAux, int kMult, int kShape>
+__global__ void __launch_bounds__(kHalfThreads, kShape == kTile32 ? (kAux ? 6 : 7) : (kAux ? 7 : 8))
 composite_px_kernel(const CompositeParams *__restrict__ pp, const float *__restrict__ rec, int n,
                     const uint2 *__restrict__ ranges, const uint32_t *__restrict__ kept,
                     const uint32_t *__restrict__ vals, const uint32_t *__restrict__ items,
@@ -872,7 +641,7 @@ composite_px_kernel(const CompositeParams *__restrict__ pp, const float *__restr
                     uint32_t *__restrict__ n_contrib, float *__restrict__ depth,
                     unsigned long long *__restrict__ counters) {
   pdl_begin();
-  __shared__ HalfSmem<kMult> sm;
+  __shared__ ItemSmem<kMult> sm;
   const CompositeParams &p = *pp;
   float *out = p.out;
   const int t = threadIdx.x, lane = t & 31;
@@ -904,14 +673,15 @@ composite_px_kernel(const CompositeParams *__restrict__ pp, const float *__restr
     range.x = min(range.x, n_kept);
     range.y = min(range.y, n_kept);
     const bool inherit = !incremental && lo == 0 && hi < 4;
+    constexpr int TS = kShape == kTile32 ? 32 : 16;
+    const int eye = gtile / p.n_tiles;
+    const int tile = gtile - eye * p.n_tiles;
+    const int tx = tile % p.tiles_x, ty = tile / p.tiles_x;
     if (range.y <= range.x) {
       // no Gaussian reaches the tile: background (0) for every pixel the tile's items would
       // write (this is the tile's only item)
-      const int eye = gtile / p.n_tiles;
-      const int tile = gtile - eye * p.n_tiles;
-      const int tx = tile % p.tiles_x, ty = tile / p.tiles_x;
-      for (int b = t; b < 256; b += kHalfThreads) {
-        const int px0 = tx * 32 + 2 * (b & 15), py0 = ty * 32 + 2 * (b >> 4);
+      for (int b = t; b < TS * TS / 4; b += kHalfThreads) {
+        const int px0 = tx * TS + 2 * (b % (TS / 2)), py0 = ty * TS + 2 * (b / (TS / 2));
         for (int L = lo; L < 4; ++L) {
           if (L >= hi && !inherit) break;
           const int x = px0 + label_dx(L), y = py0 + label_dy(L);
@@ -928,10 +698,26 @@ composite_px_kernel(const CompositeParams *__restrict__ pp, const float *__restr
         }
       }
     } else {
-#define A3FR_HALF(PP, LO0) \
-  render_half<PP, kAux, kMult, LO0>(sm, p, rec, n, range, gtile, half, lo, inherit, vals, t_final, \
-                                    n_contrib, depth, ev, bl, staged)
-      if (lo == 0) {
+      int px0, py0;
+#define A3FR_RENDER(PP, INHERIT, HI)                                                                             \
+  render_pixels<PP, kAux, kMult>(sm, p, rec, n, eye, range, lp, INHERIT, HI, px0, py0, vals, t_final, n_contrib, \
+                                 depth, ev, bl, staged)
+#define A3FR_HALF(PP, LO0)                                            \
+  {                                                                   \
+    const auto lp = pixels32<PP, LO0>(p, tx, ty, half, lo, px0, py0); \
+    A3FR_RENDER(PP, inherit, LO0 ? PP : hi);                          \
+  }
+      if constexpr (kShape != kTile32) {
+        // the lanes of slot 0 hold label lo
+        const bool mine = inherit && lane < (kShape == kTile16 ? 16 : 8);
+        if (kShape == kTile16 && P > 2) {
+          const auto lp = pixels16<2, 4>(p, tx, ty, half, lo, P, px0, py0);
+          A3FR_RENDER(2, mine, hi);
+        } else {
+          const auto lp = pixels16<1, kShape == kTile16 ? 4 : 2>(p, tx, ty, half, lo, P, px0, py0);
+          A3FR_RENDER(1, mine, hi);
+        }
+      } else if (lo == 0) {
         switch (P) {
           case 1: A3FR_HALF(1, true); break;
           case 2: A3FR_HALF(2, true); break;
@@ -946,6 +732,7 @@ composite_px_kernel(const CompositeParams *__restrict__ pp, const float *__restr
         }
       }
 #undef A3FR_HALF
+#undef A3FR_RENDER
     }
     __syncthreads();   // every thread has read sm.item and is done with the staging arrays
   }
@@ -967,9 +754,8 @@ composite_px_kernel(const CompositeParams *__restrict__ pp, const float *__restr
 
 }  // namespace
 
-// The plan buffer: the 16-pixel path's buckets [4 * n_ranges] and counts [4] at its start,
-// the 32-pixel path's items [kItemClasses * 4 * n_ranges], then its class counts
-// [kItemClasses] and work counter.
+// The plan buffer: the items [kItemClasses * 4 * n_ranges], then their class counts [kItemClasses]
+// and the work counter.
 size_t plan_bytes(int n_ranges) {
   return sizeof(uint32_t) * ((size_t)kItemClasses * 4 * (size_t)n_ranges + kItemClasses + 8);
 }
@@ -1008,80 +794,45 @@ cudaError_t launch_composite(const CompositeParams &p, const CompositeParams *p_
     if (e != cudaSuccess) return e;
     if (kernels) ++*kernels;
   }
-  if (p.tile == 32) {
-    // plan (every tile, also for the full render: uniform level 4) + one persistent composite
-    uint32_t *items = plan;
-    uint32_t *class_counts = plan + (size_t)kItemClasses * 4 * n_ranges;
-    uint32_t *work = class_counts + kItemClasses;
-    cudaError_t e = cudaMemsetAsync(class_counts, 0, sizeof(uint32_t) * (kItemClasses + 1), s);
-    if (e != cudaSuccess) return e;
-    {
-      const cudaError_t e_ = launch_pdl(plan32_kernel, (n_ranges + 255) / 256, 256, 0, s, p_dev, gaze, round,
-                                        p.full ? 4 : uniform, cur, levels, items, class_counts, ranges,
-                                        thresholds);
-      if (e_ != cudaSuccess) return e_;
+  // plan (every tile, also for the full render: uniform level 4) + one persistent composite
+  uint32_t *items = plan;
+  uint32_t *class_counts = plan + (size_t)kItemClasses * 4 * n_ranges;
+  uint32_t *work = class_counts + kItemClasses;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
+  const int shape = p.tile == 32 ? kTile32 : (n_ranges <= kSplitTilesPerSm * sms ? kTile16Split : kTile16);
+  const int parts = shape == kTile16 ? 1 : 2;
+  cudaError_t e = cudaMemsetAsync(class_counts, 0, sizeof(uint32_t) * (kItemClasses + 1), s);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(plan_kernel, (n_ranges + 255) / 256, 256, 0, s, p_dev, gaze, round, p.full ? 4 : uniform, parts, cur,
+                 levels, items, class_counts, ranges, thresholds);
+  if (e != cudaSuccess) return e;
+  auto go = [&](auto kern, int variant) -> cudaError_t {
+    prefer_smem(kern, variant);
+    static int per_sm[64][16] = {};
+    int occ = (dev >= 0 && dev < 64) ? per_sm[dev][variant] : 0;
+    if (occ == 0) {
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kHalfThreads, 0) != cudaSuccess || occ < 1)
+        occ = 1;
+      if (dev >= 0 && dev < 64) per_sm[dev][variant] = occ;
     }
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    auto go = [&](auto kern, int variant) -> cudaError_t {
-      prefer_smem(kern, variant);
-      static int per_sm[64][16] = {};
-      int dev = 0;
-      cudaGetDevice(&dev);
-      int occ = (dev >= 0 && dev < 64) ? per_sm[dev][variant] : 0;
-      int sms = 0;
-      if (occ == 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kHalfThreads, 0) != cudaSuccess || occ < 1)
-          occ = 1;
-        if (dev >= 0 && dev < 64) per_sm[dev][variant] = occ;
-      }
-      if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        sms = 1;
-      const long max_items = 2L * n_ranges;
-      const int grid = (int)std::min<long>((long)sms * occ, max_items);
-      {
-        const cudaError_t e_ = launch_pdl(kern, grid, kHalfThreads, 0, s, p_dev, rec, n, ranges, kept, vals,
-                                          items, class_counts, work, inc, t_final, n_contrib, depth,
-                                          counters);
-        if (e_ != cudaSuccess) return e_;
-      }
-      return cudaGetLastError();
-    };
-    e = aux ? (mult == 2 ? go(composite_px_kernel<true, 2>, 0) : go(composite_px_kernel<true, 1>, 1))
-            : (mult == 2 ? go(composite_px_kernel<false, 2>, 2) : go(composite_px_kernel<false, 1>, 3));
-    if (kernels) *kernels += 2;
-    return e;
-  }
-  uint32_t *pc = plan + 4 * (size_t)n_ranges;
-  if (!p.full) {
-    cudaError_t e = cudaMemsetAsync(pc, 0, 4 * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
-    {
-      const cudaError_t e_ = launch_pdl(plan_kernel, (n_ranges + 255) / 256, 256, 0, s, p_dev, gaze, round,
-                                        uniform, cur, levels, plan, pc, ranges, thresholds);
-      if (e_ != cudaSuccess) return e_;
-    }
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (kernels) ++*kernels;
-  }
-  auto launch = [&](auto kern, int variant) -> cudaError_t {
-    prefer_smem(kern, 4 + variant);
-    {
-      const cudaError_t e_ = launch_pdl(kern, n_ranges, kThreads, 0, s, p_dev, rec, n, ranges, kept, vals,
-                                        plan, pc, p.full ? 0 : inc, levels, t_final, n_contrib, depth,
-                                        counters);
-      if (e_ != cudaSuccess) return e_;
-    }
-    if (kernels) ++*kernels;
-    return cudaGetLastError();
+    const int grid = (int)std::min<long>((long)sms * occ, (long)parts * n_ranges);
+    return launch_pdl(kern, grid, kHalfThreads, 0, s, p_dev, rec, n, ranges, kept, vals, items, class_counts, work,
+                      inc, t_final, n_contrib, depth, counters);
   };
-  if (aux) {
-    if (p.full) return mult == 2 ? launch(composite_kernel<true, true, 2>, 0) : launch(composite_kernel<true, true, 1>, 1);
-    return mult == 2 ? launch(composite_kernel<true, false, 2>, 2) : launch(composite_kernel<true, false, 1>, 3);
+  if (kernels) *kernels += 2;
+  switch (shape) {
+    case kTile32:
+      return aux ? (mult == 2 ? go(composite_px_kernel<true, 2, kTile32>, 0) : go(composite_px_kernel<true, 1, kTile32>, 1))
+                 : (mult == 2 ? go(composite_px_kernel<false, 2, kTile32>, 2) : go(composite_px_kernel<false, 1, kTile32>, 3));
+    case kTile16:
+      return aux ? (mult == 2 ? go(composite_px_kernel<true, 2, kTile16>, 4) : go(composite_px_kernel<true, 1, kTile16>, 5))
+                 : (mult == 2 ? go(composite_px_kernel<false, 2, kTile16>, 6) : go(composite_px_kernel<false, 1, kTile16>, 7));
+    default:
+      return aux ? (mult == 2 ? go(composite_px_kernel<true, 2, kTile16Split>, 8) : go(composite_px_kernel<true, 1, kTile16Split>, 9))
+                 : (mult == 2 ? go(composite_px_kernel<false, 2, kTile16Split>, 10) : go(composite_px_kernel<false, 1, kTile16Split>, 11));
   }
-  if (p.full) return mult == 2 ? launch(composite_kernel<false, true, 2>, 4) : launch(composite_kernel<false, true, 1>, 5);
-  return mult == 2 ? launch(composite_kernel<false, false, 2>, 6) : launch(composite_kernel<false, false, 1>, 7);
 }
 
 }  // namespace a3fr
