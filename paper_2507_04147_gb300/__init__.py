@@ -232,7 +232,8 @@ def get_round_status(handle: int) -> dict:
 def run_frame(handle: int, fovea, rounds, predictions, exit_time_us, out_rgb, mode: int = 0,
               load_period_us: float = 0.0, load_factor: float = 1.0, max_rounds: int = 64,
               stream=None) -> dict:
-    """One frame of Algorithm 1 in native code (see a3fr_run_frame)."""
+    """One frame of Algorithm 1 in native code (see a3fr_run_frame).  "exits" is the exit consumed
+    by each of the first 16 rounds and, when there were more, by the last one."""
     pred = np.ascontiguousarray(np.asarray(predictions, dtype=np.float32))
     times = np.ascontiguousarray(np.asarray(exit_time_us, dtype=np.float64))
     d = _lib.FrameDriver()
@@ -244,8 +245,9 @@ def run_frame(handle: int, fovea, rounds, predictions, exit_time_us, out_rgb, mo
                                           ctypes.byref(d), _ptr(out_rgb), _stream_ptr(stream),
                                           ctypes.byref(r)), "a3fr_run_frame")
     k = min(r.rounds, 16)
+    last = [get_round_status(handle)["exit_consumed"]] if r.rounds > 16 else []
     return {"latency_us": r.latency_us, "tracker_end_us": r.tracker_end_us, "rounds": r.rounds,
-            "exits": list(r.exit_per_round[:k]), "round_end_us": list(r.round_end_us[:k])}
+            "exits": list(r.exit_per_round[:k]) + last, "round_end_us": list(r.round_end_us[:k])}
 
 
 def error_string(code: int) -> str:
