@@ -230,7 +230,7 @@ __device__ __forceinline__ bool falloff_reaches(float A, float B, float C, float
 //   kTile16       16-pixel tiles: an item is a tile, a warp's patch 8 x 8 pixels, two pixels a lane.
 //                 Bound by issue, as kTile32; every warp walking the whole list of its tile, one
 //                 pixel a lane, took 254 us on the 1M-Gaussian 1920 x 1080 full render (ncu), this
-//                 shape 117 us.
+//                 shape 111 us.
 //   kTile16Split  the same in half tiles, a patch 8 x 4 pixels, one pixel a lane: for renders with
 //                 too few tiles to fill the device, which are bound by the longest list's chain of
 //                 blends; fewer Gaussians reach the smaller patch.
@@ -281,12 +281,14 @@ __device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
 
 template <int kMult>
 struct ItemSmem {
-  float4 geo[kBatch * kMult];
-  float2 cz[kBatch * kMult];
-  float4 rgb[kBatch * kMult];
+  // one slot past the batch: a Gaussian of opacity 0, which fails the 1/255 test everywhere
+  float4 geo[kBatch * kMult + 1];
+  float2 cz[kBatch * kMult + 1];
+  float4 rgb[kBatch * kMult + 1];
   short4 box[kBatch * kMult];        // support box, outward-rounded pixels
   float thr[kBatch * kMult];         // log2 falloff needed for alpha = 1/255
-  uint16_t hits[kHalfThreads / 32][kBatch * kMult];   // per warp: batch slots that reach its patch
+  // per warp: batch slots that reach its patch, padded to a multiple of 4 with the empty slot
+  uint16_t hits[kHalfThreads / 32][kBatch * kMult + 4];
   int done[kHalfThreads / 32];
   uint32_t prefix[kItemClasses + 1];  // item index ranges, heaviest class first
   uint32_t item;
@@ -399,13 +401,18 @@ __device__ __forceinline__ void render_pixels(ItemSmem<kMult> &sm, const Composi
           n_keep += __popc(m);
         }
         n_hit = n_keep;
+        // padding: the steps of four below have no exit inside them, so their loads overlap
+        // (with one after each: 500k stereo composite 107 -> 99 us, the longest chain of the 20k
+        // 256 x 256 view 96 -> 75 us)
+        if (lane < 3) sm.hits[warp][n_hit + lane] = (uint16_t)NB;
       }
       __syncwarp();
       const uint32_t pos0 = start - range.x + 1;
       for (int i = 0; i < n_hit; i += 4) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          if (i + j >= n_hit) break;
+          // four of these at once would spill (248 bytes; 500k stereo frame 407 -> 425 us)
+          if (kAux && P > 2 && i + j >= n_hit) break;
           const int e = sm.hits[warp][i + j];
           const float4 geo = sm.geo[e];
           const float2 cz = sm.cz[e];
@@ -632,7 +639,7 @@ __device__ __forceinline__ LanePixels<Q> pixels16(const CompositeParams &p, int 
 }
 
 template <bool kAux, int kMult, int kShape>
-__global__ void __launch_bounds__(kHalfThreads, kShape == kTile32 ? (kAux ? 6 : 7) : (kAux ? 7 : 8))
+__global__ void __launch_bounds__(kHalfThreads, kAux ? 6 : 7)
 composite_px_kernel(const CompositeParams *__restrict__ pp, const float *__restrict__ rec, int n,
                     const uint2 *__restrict__ ranges, const uint32_t *__restrict__ kept,
                     const uint32_t *__restrict__ vals, const uint32_t *__restrict__ items,
@@ -648,6 +655,9 @@ composite_px_kernel(const CompositeParams *__restrict__ pp, const float *__restr
   const int n_ranges = p.n_eyes * p.n_tiles;
   const size_t cap = 4 * (size_t)n_ranges;
   if (t == 0) {
+    sm.geo[kBatch * kMult] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    sm.cz[kBatch * kMult] = make_float2(0.0f, 0.0f);
+    sm.rgb[kBatch * kMult] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     sm.prefix[0] = 0u;
     for (int i = 0; i < kItemClasses; ++i)
       sm.prefix[i + 1] = sm.prefix[i] + class_counts[kItemClasses - 1 - i];
