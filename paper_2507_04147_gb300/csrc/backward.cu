@@ -2,195 +2,299 @@
 // with respect to the scene parameters, for a loss whose gradient with respect to the
 // rendered image is given (L = sum(dl_drgb * image)).
 //
-// composite_backward: one CTA per 16 x 16 quadrant of an (eye, tile), one pixel per thread.  A pixel walks its
-// tile's Gaussians back to front from its last contributor (n_contrib), recovering the
+// composite_backward: one CTA per 16 x 16 quadrant of an (eye, tile), or per half of one.  A pixel
+// walks its tile's Gaussians back to front from its last contributor (n_contrib), recovering the
 // transmittance before each contributor from the stored final one (T_before = T_after /
 // (1 - alpha)) instead of storing it per Gaussian.  The colour accumulated behind a
 // contributor enters the alpha gradient only through its dot product with dL/dC, so one
 // scalar D carries it:  dL/dalpha_i = T_i (c_i . g - D_i),  D_{i-1} = alpha_i c_i . g +
 // (1 - alpha_i) D_i.  Alpha is recomputed exactly as the forward computed it (shared
-// helpers, explicitly rounded), so every skip / accept decision is the forward's.  The
-// per-Gaussian partials (2-D mean, conic, opacity, colour) are summed over the warp and
-// added to a per-(eye, Gaussian) buffer with one atomic per warp and value.  A foveated
-// render's inherited pixels pass their gradient to the top-left pixel of their block.
+// helpers, explicitly rounded), so every skip / accept decision is the forward's.  Nine sums over
+// the pixels -- w g (three), dL/dopacity, and with p = dL/dpower those of p dx, p dy, p dx^2,
+// p dx dy, p dy^2 -- go to a per-(eye, Gaussian) buffer; what is linear in the conic is left to
+// preprocess_backward.  A foveated render's inherited pixels pass their gradient to the top-left
+// pixel of their block.
 //
 // preprocess_backward: one thread per Gaussian, summing the eyes: conic -> 2-D covariance
 // -> (3-D covariance, Jacobian) -> camera-space position -> mean; 3-D covariance ->
 // scales (through exp) and rotation -> quaternion (through the normalisation); opacity
 // through the sigmoid; colour -> SH coefficients and, through the view direction, mean.
+#include "blend.cuh"
 #include "common.cuh"
 
 namespace a3fr {
 namespace {
 
 constexpr int kTile = 16;
-constexpr int kThreads = 256;
-constexpr int kG2 = 9;   // per (eye, Gaussian): du dv dconic_a dconic_b dconic_c dopacity dr dg db
+constexpr int kThreads = 128;            // four warps
+constexpr int kBatch = 128;              // Gaussians staged per batch
+constexpr int kG2 = 9;                   // sums per (eye, Gaussian): eight side by side, the ninth apart
 constexpr int kPreBwdThreads = 128;
+// Quadrants are split in halves up to this many per SM, as the forward's 16-pixel tiles are: split /
+// not, 825 quadrants 102 / 145 us, 4,096 quadrants 160 / 146 us (ncu).
+constexpr int kSplitQuadsPerSm = 16;
 
-__global__ void __launch_bounds__(kThreads)
+// Where the sums of (eye, Gaussian) entry q of n_entries lie: [n_entries][8] -- p dx, p dy, p dx^2,
+// p dx dy, p dy^2, dopacity, dr, dg (one 32-byte sector) -- then [n_entries] db.
+__device__ __forceinline__ float *sums8(float *g2d, size_t q) { return g2d + 8 * q; }
+__device__ __forceinline__ float *sum9(float *g2d, size_t q, size_t n_entries) { return g2d + 8 * n_entries + q; }
+
+// Each warp owns a patch of 8 x 8 pixels (Q = 2: lanes are 4 x 4 blocks of 2 x 2 pixels times two
+// label pairs) or of 8 x 4 (Q = 1: 4 x 2 blocks times four labels); per batch it lists the
+// Gaussians that can reach alpha = 1/255 in its patch (falloff_reaches: the others contribute to no
+// pixel of it) and walks only those, two at a time, so that the warp sums of one overlap the
+// other's.  The sums of a batch meet in shared memory, one row per warp and Gaussian, and leave as
+// one reduction per value, Gaussian and quadrant.
+// Bound by issue, and by the longest list's chain on small images.  1M Gaussians at 1024 x 1024 (ncu):
+// 281 us with every warp (16 x 2 pixels) walking the whole list and adding its own nine sums to
+// memory, 146 us now; 50k at 517 x 389: 247, 102 us.
+template <int Q>
+__global__ void __launch_bounds__(kThreads, 6)
 composite_backward_kernel(BackwardParams p, const float *__restrict__ rec, const uint2 *__restrict__ ranges,
                           const uint32_t *__restrict__ kept, const uint32_t *__restrict__ vals,
                           const uint8_t *__restrict__ levels, const float *__restrict__ t_final,
                           const uint32_t *__restrict__ n_contrib, const float *__restrict__ dl_drgb,
                           float *__restrict__ g2d) {
-  __shared__ float4 s_geo[kThreads];   // u, v, A, B (base-2 falloff coefficients)
-  __shared__ float4 s_cn[kThreads];    // C, conic a, conic b, conic c
-  __shared__ float4 s_rgb[kThreads];   // r, g, b, opacity
-  __shared__ uint32_t s_gid[kThreads];
-  __shared__ uint32_t s_max[kThreads / 32];
+  constexpr int BH = Q == 2 ? 4 : 2;   // blocks down a patch
+  constexpr int W = kThreads / 32;
+  // slot kBatch: a Gaussian of opacity 0, which pads odd hit lists
+  __shared__ float4 s_geo[kBatch + 1];   // u, v, A, B (base-2 falloff coefficients)
+  __shared__ float4 s_crg[kBatch + 1];   // C, opacity, r, g
+  __shared__ float s_b[kBatch + 1];
+  __shared__ uint32_t s_gid[kBatch];
+  __shared__ short4 s_box[kBatch];
+  __shared__ float s_thr[kBatch];
+  __shared__ uint8_t s_hits[W][kBatch + 4];
+  __shared__ uint32_t s_mask[W][kBatch / 32];   // slots with sums of this warp
+  __shared__ float s_sum[W][kBatch + 1][kG2];
+  __shared__ uint32_t s_max[W];
 
-  // one CTA per 16 x 16 quadrant of a tile (a 16-pixel tile is one quadrant, a 32-pixel tile
-  // four, each walking the tile's whole list for its own pixels)
-  const int qn = p.tile / kTile;
-  const int gtile = blockIdx.x / (qn * qn);
-  const int quad = blockIdx.x - gtile * qn * qn;
+  const int qn = p.tile / kTile, parts = Q == 2 ? 1 : 2;
+  const int gtile = blockIdx.x / (qn * qn * parts);
+  const int rest = blockIdx.x - gtile * qn * qn * parts, quad = rest / parts, half = rest - quad * parts;
   const int eye = gtile / p.n_tiles;
   const int tile = gtile - eye * p.n_tiles;
   const int tx = tile % p.tiles_x, ty = tile / p.tiles_x;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int px = tx * p.tile + (quad % qn) * kTile + (t & 15);
-  const int py = ty * p.tile + (quad / qn) * kTile + (t >> 4);
-  const bool inside = px < p.width && py < p.height;
-  // labels of the 2x2 block: top-left 0, bottom-right 1, top-right 2, bottom-left 3
-  const int bx = px & 1, by = py & 1;
-  const int lab = bx == by ? (bx ? 1 : 0) : (bx ? 2 : 3);
+  const int wx = tx * p.tile + (quad % qn) * kTile + 8 * (warp & 1);
+  const int wy = ty * p.tile + (quad / qn) * kTile + (Q == 2 ? 0 : 8 * half) + 2 * BH * (warp >> 1);
+  const int blk = lane % (4 * BH), slot0 = lane / (4 * BH) * Q;
+  const int px0 = wx + 2 * (blk & 3), py0 = wy + 2 * (blk >> 2);
   const int level = levels ? levels[gtile] : 4;
-  const bool rendered = inside && lab < level;
-
-  float T = 1.0f, g0 = 0.0f, g1 = 0.0f, g2 = 0.0f;
-  uint32_t last = 0;
-  if (rendered) {
-    const size_t pix = ((size_t)eye * p.height + py) * p.width + px;
-    T = t_final[pix];
-    last = n_contrib[pix];
-    g0 = dl_drgb[3 * pix];
-    g1 = dl_drgb[3 * pix + 1];
-    g2 = dl_drgb[3 * pix + 2];
-    if (lab == 0 && level < 4) {
-      // inherited pixels of the block copy this one: BR (label 2), TR (label 3), BL (label 4)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const int dx = k < 2 ? 1 : 0, dy = k == 1 ? 0 : 1;
-        if (level < k + 2 && px + dx < p.width && py + dy < p.height) {
-          const size_t q = pix + (size_t)dy * p.width + dx;
-          g0 += dl_drgb[3 * q];
-          g1 += dl_drgb[3 * q + 1];
-          g2 += dl_drgb[3 * q + 2];
-        }
-      }
-    }
-  }
   uint2 range = ranges[gtile];
   const uint32_t n_kept = *kept;
   range.x = min(range.x, n_kept);
   range.y = min(range.y, n_kept);
-  last = min(last, range.y - range.x);
 
-  // the block's deepest last contributor bounds the walk
-  uint32_t m = last;
+  float T[Q], D[Q], g[Q][3], fpx[Q], fpy[Q];   // D: colour accumulated behind, normalised by T, . dL/dC
+  uint32_t last[Q];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) s_max[warp] = m;
+  for (int k = 0; k < Q; ++k) {
+    // labels of the 2x2 block: top-left 0, bottom-right 1, top-right 2, bottom-left 3
+    const int L = slot0 + k;
+    const int px = px0 + ((L == 1 || L == 2) ? 1 : 0), py = py0 + ((L == 1 || L == 3) ? 1 : 0);
+    fpx[k] = (float)px;
+    fpy[k] = (float)py;
+    T[k] = 1.0f;
+    D[k] = g[k][0] = g[k][1] = g[k][2] = 0.0f;
+    last[k] = 0u;
+    if (L < level && px < p.width && py < p.height) {
+      const size_t pix = ((size_t)eye * p.height + py) * p.width + px;
+      T[k] = t_final[pix];
+      last[k] = min(n_contrib[pix], range.y - range.x);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) g[k][c] = dl_drgb[3 * pix + c];
+      if (L == 0 && level < 4) {
+        // inherited pixels of the block copy this one: BR (label 2), TR (label 3), BL (label 4)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const int dx = j < 2 ? 1 : 0, dy = j == 1 ? 0 : 1;
+          if (level < j + 2 && px + dx < p.width && py + dy < p.height) {
+            const size_t q = pix + (size_t)dy * p.width + dx;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) g[k][c] += dl_drgb[3 * q + c];
+          }
+        }
+      }
+    }
+  }
+  // the deepest last contributor bounds the walk: the warp's for its lists, the CTA's for the batches
+  uint32_t wlast = last[0];
+  if (Q == 2) wlast = max(wlast, last[Q - 1]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) wlast = max(wlast, __shfl_xor_sync(0xffffffffu, wlast, o));
+  if (lane == 0) s_max[warp] = wlast;
+  if (t == 0) {
+    s_geo[kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    s_crg[kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    s_b[kBatch] = 0.0f;
+  }
   __syncthreads();
   uint32_t max_last = 0;
 #pragma unroll
-  for (int w = 0; w < kThreads / 32; ++w) max_last = max(max_last, s_max[w]);
+  for (int w = 0; w < W; ++w) max_last = max(max_last, s_max[w]);
 
-  const float fpx = (float)px, fpy = (float)py;
+  const float wx0 = (float)wx, wx1 = (float)(wx + 7), wy0 = (float)wy, wy1 = (float)(wy + 2 * BH - 1);
   const float *rec_eye = rec + (size_t)eye * p.n * kRec;
-  float *g_eye = g2d + (size_t)eye * p.n * kG2;
-  float D = 0.0f;   // (colour accumulated behind, normalised by T) . dL/dC
+  const size_t n_entries = (size_t)p.n_eyes * p.n, q0 = (size_t)eye * p.n;
 
-  for (int hi = (int)max_last; hi >= 1; hi -= kThreads) {
-    const int lo = max(1, hi - kThreads + 1);
-    const int cnt = hi - lo + 1;
-    __syncthreads();   // the previous batch is no longer read
+  for (int hi = (int)max_last; hi >= 1; hi -= kBatch) {
+    const int cnt = min(hi, kBatch);   // slot k: 1-based position hi - k of the tile's list
+    __syncthreads();                   // the previous batch's sums have left
     if (t < cnt) {
-      const uint32_t pos = (uint32_t)(hi - t);   // 1-based position in the tile's list
-      const uint32_t gidx = min(vals[range.x + pos - 1], (uint32_t)(p.n - 1));
+      const uint32_t gidx = min(vals[range.x + (uint32_t)(hi - t) - 1u], (uint32_t)(p.n - 1));
       const float4 *r4 = reinterpret_cast<const float4 *>(rec_eye + (size_t)gidx * kRec);
-      const float4 a = __ldg(r4), b = __ldg(r4 + 1), c = __ldg(r4 + 2);
+      const float4 a = __ldg(r4), b = __ldg(r4 + 1);
       s_geo[t] = make_float4(a.x, a.y, __fmul_rn(-0.5f * kLog2e, a.z), __fmul_rn(-kLog2e, a.w));
-      s_cn[t] = make_float4(__fmul_rn(-0.5f * kLog2e, b.x), a.z, a.w, b.x);
-      s_rgb[t] = make_float4(b.z, b.w, c.x, b.y);
+      s_crg[t] = make_float4(__fmul_rn(-0.5f * kLog2e, b.x), b.y, b.z, b.w);
+      s_b[t] = __ldg(rec_eye + (size_t)gidx * kRec + 8);
       s_gid[t] = gidx;
+      s_box[t] = int_box(support_box(a.x, a.y, a.z, a.w, b.x, b.y));
+      s_thr[t] = -__log2f(255.0f * b.y) - 0.01f;
     }
     __syncthreads();
-    for (int k = 0; k < cnt; ++k) {
-      const uint32_t pos = (uint32_t)(hi - k);
-      const float4 geo = s_geo[k];
-      const float4 cn = s_cn[k];
-      const float4 rgb = s_rgb[k];
-      float vu = 0.f, vv = 0.f, va = 0.f, vb = 0.f, vc = 0.f, vo = 0.f, vr = 0.f, vg = 0.f, vbl = 0.f;
-      bool ok = false;
-      if (pos <= last) {
-        const float dx = __fsub_rn(geo.x, fpx), dy = __fsub_rn(geo.y, fpy);
-        const float pw = falloff_log2(geo.z, geo.w, cn.x, dx, dy);
-        const float G = ex2_approx(pw);
-        const float araw = __fmul_rn(rgb.w, G);
-        const float alpha = fminf(0.99f, araw);
-        ok = pw <= 0.0f && alpha >= 1.0f / 255.0f;
-        if (ok) {
-          const float om = __fsub_rn(1.0f, alpha);
-          T = T / om;                              // transmittance in front of this Gaussian
-          const float w = alpha * T;
-          vr = w * g0;
-          vg = w * g1;
-          vbl = w * g2;
-          const float cdot = rgb.x * g0 + rgb.y * g1 + rgb.z * g2;
-          const float dalpha = T * (cdot - D);
-          D = alpha * cdot + om * D;
-          if (araw <= 0.99f) {                     // the 0.99 clamp passes no gradient
-            const float dpow = dalpha * araw;      // d alpha / d power = opacity * exp(power)
-            vo = dalpha * G;
-            // power = -0.5 (a dx^2 + c dy^2) - b dx dy with dx = u - x, dy = v - y
-            vu = -dpow * (cn.y * dx + cn.z * dy);
-            vv = -dpow * (cn.w * dy + cn.z * dx);
-            va = -0.5f * dpow * dx * dx;
-            vb = -dpow * dx * dy;
-            vc = -0.5f * dpow * dy * dy;
-          }
+    int n_hit = 0;
+    for (int base = 0; base < kBatch; base += 32) {
+      const int k = base + lane;
+      bool hit = k < cnt && hi - k <= (int)wlast;
+      if (hit) {
+        const short4 box = s_box[k];
+        hit = !((float)box.y < wx0 || (float)box.x > wx1 || (float)box.w < wy0 || (float)box.z > wy1);
+        if (hit) {
+          const float4 geo = s_geo[k];
+          hit = falloff_reaches(geo.z, geo.w, s_crg[k].x, s_thr[k], wx0 - geo.x, wx1 - geo.x, wy0 - geo.y,
+                                wy1 - geo.y);
         }
       }
-      if (__ballot_sync(0xffffffffu, ok)) {
-        // warp sums of the nine partials by recursive halving: at each of the first three
-        // steps a lane keeps half of its values and sends the other half to its partner, so
-        // the first eight cost 4 + 2 + 1 + 1 + 1 shuffles instead of 8 x 5; value j ends in
-        // the lanes whose bits 4, 3, 2 spell j, and eight lanes add them to memory at once
-        float h[8] = {vu, vv, va, vb, vc, vo, vr, vg};
-        {
-          const bool up = (lane & 16) != 0;
+      const unsigned m = __ballot_sync(0xffffffffu, hit);
+      if (hit) s_hits[warp][n_hit + __popc(m & ((1u << lane) - 1u))] = (uint8_t)k;
+      if (lane == 0) s_mask[warp][base / 32] = m;
+      n_hit += __popc(m);
+    }
+    if (lane == 0) s_hits[warp][n_hit] = (uint8_t)kBatch;
+    __syncwarp();
+    for (int i = 0; i < n_hit; i += 2) {
+      float v[2][kG2];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float keep = up ? h[j + 4] : h[j], send = up ? h[j] : h[j + 4];
-            h[j] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-          }
-        }
-        {
-          const bool up = (lane & 8) != 0;
+      for (int u = 0; u < 2; ++u) {
+        const int e = s_hits[warp][i + u];
+        const float4 geo = s_geo[e], crg = s_crg[e];
+        const float cb = s_b[e];
+        const uint32_t pos = (uint32_t)(hi - e);
 #pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const float keep = up ? h[j + 2] : h[j], send = up ? h[j] : h[j + 2];
-            h[j] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-          }
+        for (int j = 0; j < kG2; ++j) v[u][j] = 0.0f;
+        if constexpr (Q == 2) {
+          // both pixels per instruction where the arithmetic is the same
+          const f32x2 dx = f2_add(f2_pack(geo.x, geo.x), f2_pack(-fpx[0], -fpx[Q - 1]));
+          const f32x2 dy = f2_add(f2_pack(geo.y, geo.y), f2_pack(-fpy[0], -fpy[Q - 1]));
+          const f32x2 pw = f2_fma(f2_fma(f2_pack(geo.z, geo.z), dx, f2_mul(f2_pack(geo.w, geo.w), dy)), dx,
+                                  f2_mul(f2_mul(f2_pack(crg.x, crg.x), dy), dy));
+          float pw0, pw1, ar0, ar1;
+          f2_unpack(pw, pw0, pw1);
+          const float G0 = ex2_approx(pw0), G1 = ex2_approx(pw1);
+          f2_unpack(f2_mul(f2_pack(crg.y, crg.y), f2_pack(G0, G1)), ar0, ar1);
+          const float al0 = fminf(0.99f, ar0), al1 = fminf(0.99f, ar1);
+          const bool ok0 = pos <= last[0] && pw0 <= 0.0f && al0 >= 1.0f / 255.0f;
+          const bool ok1 = pos <= last[Q - 1] && pw1 <= 0.0f && al1 >= 1.0f / 255.0f;
+          // a pixel this Gaussian does not touch takes alpha 0: T and D keep their bits
+          const float a0 = ok0 ? al0 : 0.0f, a1 = ok1 ? al1 : 0.0f;
+          const bool free0 = ok0 && ar0 <= 0.99f, free1 = ok1 && ar1 <= 0.99f;   // the clamp passes no gradient
+          const f32x2 a2 = f2_pack(a0, a1), om = f2_pack(__fsub_rn(1.0f, a0), __fsub_rn(1.0f, a1));
+          T[0] = T[0] / __fsub_rn(1.0f, a0);   // transmittance in front of this Gaussian
+          T[Q - 1] = T[Q - 1] / __fsub_rn(1.0f, a1);
+          const f32x2 T2 = f2_pack(T[0], T[Q - 1]), D2 = f2_pack(D[0], D[Q - 1]);
+          const f32x2 g0 = f2_pack(g[0][0], g[Q - 1][0]), g1 = f2_pack(g[0][1], g[Q - 1][1]),
+                      g2 = f2_pack(g[0][2], g[Q - 1][2]);
+          const f32x2 w2 = f2_mul(a2, T2);
+          const f32x2 cdot = f2_fma(f2_pack(crg.z, crg.z), g0,
+                                    f2_fma(f2_pack(crg.w, crg.w), g1, f2_mul(f2_pack(cb, cb), g2)));
+          const f32x2 dal = f2_mul(T2, f2_fma(D2, f2_pack(-1.0f, -1.0f), cdot));
+          f2_unpack(f2_fma(a2, cdot, f2_mul(om, D2)), D[0], D[Q - 1]);
+          const f32x2 dpow = f2_mul(dal, f2_pack(free0 ? ar0 : 0.0f, free1 ? ar1 : 0.0f));
+          const f32x2 px2 = f2_mul(dpow, dx), py2 = f2_mul(dpow, dy);
+          v[u][0] = f2_sum(px2);
+          v[u][1] = f2_sum(py2);
+          v[u][2] = f2_sum(f2_mul(px2, dx));
+          v[u][3] = f2_sum(f2_mul(px2, dy));
+          v[u][4] = f2_sum(f2_mul(py2, dy));
+          v[u][5] = f2_sum(f2_mul(dal, f2_pack(free0 ? G0 : 0.0f, free1 ? G1 : 0.0f)));
+          v[u][6] = f2_sum(f2_mul(w2, g0));
+          v[u][7] = f2_sum(f2_mul(w2, g1));
+          v[u][8] = f2_sum(f2_mul(w2, g2));
+        } else {
+          const float dx = __fsub_rn(geo.x, fpx[0]), dy = __fsub_rn(geo.y, fpy[0]);
+          const float pw = falloff_log2(geo.z, geo.w, crg.x, dx, dy);
+          const float G = ex2_approx(pw);
+          const float araw = __fmul_rn(crg.y, G);
+          const float al = fminf(0.99f, araw);
+          const bool ok = pos <= last[0] && pw <= 0.0f && al >= 1.0f / 255.0f;
+          const float a = ok ? al : 0.0f;
+          const bool open = ok && araw <= 0.99f;   // the clamp passes no gradient
+          const float om = __fsub_rn(1.0f, a);
+          T[0] = T[0] / om;   // transmittance in front of this Gaussian
+          const float w = a * T[0];
+          const float cdot = crg.z * g[0][0] + crg.w * g[0][1] + cb * g[0][2];
+          const float dal = T[0] * (cdot - D[0]);
+          D[0] = a * cdot + om * D[0];
+          const float dpow = dal * (open ? araw : 0.0f);
+          v[u][0] = dpow * dx;
+          v[u][1] = dpow * dy;
+          v[u][2] = v[u][0] * dx;
+          v[u][3] = v[u][0] * dy;
+          v[u][4] = v[u][1] * dy;
+          v[u][5] = dal * (open ? G : 0.0f);
+          v[u][6] = w * g[0][0];
+          v[u][7] = w * g[0][1];
+          v[u][8] = w * g[0][2];
         }
-        {
-          const bool up = (lane & 4) != 0;
-          const float keep = up ? h[1] : h[0], send = up ? h[0] : h[1];
-          h[0] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-        }
-        h[0] += __shfl_xor_sync(0xffffffffu, h[0], 2);
-        h[0] += __shfl_xor_sync(0xffffffffu, h[0], 1);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) vbl += __shfl_xor_sync(0xffffffffu, vbl, o);
-        float *d = g_eye + (size_t)s_gid[k] * kG2;
-        if ((lane & 3) == 0) {
-          const int j = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
-          atomicAdd(d + j, h[0]);
-        }
-        if (lane == 1) atomicAdd(d + 8, vbl);
       }
+      // warp sums by recursive halving: at each of the first four steps a lane keeps half of its
+      // values and sends its partner the other half, so the sixteen cost 8 + 4 + 2 + 1 + 1 shuffles;
+      // lane bit 4 ends as the Gaussian, bits 3..1 as the value; the ninth values 1 + 4
+      float h[8];
+      const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0, b2 = (lane & 4) != 0, b1 = (lane & 2) != 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        h[j] = (b4 ? v[1][j] : v[0][j]) + __shfl_xor_sync(0xffffffffu, b4 ? v[0][j] : v[1][j], 16);
+      float h9 = (b4 ? v[1][8] : v[0][8]) + __shfl_xor_sync(0xffffffffu, b4 ? v[0][8] : v[1][8], 16);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        h[j] = (b3 ? h[j + 4] : h[j]) + __shfl_xor_sync(0xffffffffu, b3 ? h[j] : h[j + 4], 8);
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+        h[j] = (b2 ? h[j + 2] : h[j]) + __shfl_xor_sync(0xffffffffu, b2 ? h[j] : h[j + 2], 4);
+      h[0] = (b1 ? h[1] : h[0]) + __shfl_xor_sync(0xffffffffu, b1 ? h[0] : h[1], 2);
+      h[0] += __shfl_xor_sync(0xffffffffu, h[0], 1);
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) h9 += __shfl_xor_sync(0xffffffffu, h9, o);
+      float *row = s_sum[warp][s_hits[warp][i + (b4 ? 1 : 0)]];
+      if (!(lane & 1)) row[(lane >> 1) & 7] = h[0];
+      else if ((lane & 15) == 1) row[8] = h9;
+    }
+    __syncthreads();
+    // the batch's sums over the warps, eight values of a Gaussian to a sector
+    for (int e = t; e < cnt * 8; e += kThreads) {
+      const int k = e >> 3, j = e & 7;
+      float sum = 0.0f;
+      bool any = false;
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        if ((s_mask[w][k >> 5] >> (k & 31)) & 1u) {
+          sum += s_sum[w][k][j];
+          any = true;
+        }
+      if (any) atomicAdd(sums8(g2d, q0 + s_gid[k]) + j, sum);
+    }
+    if (t < cnt) {
+      float sum = 0.0f;
+      bool any = false;
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        if ((s_mask[w][t >> 5] >> (t & 31)) & 1u) {
+          sum += s_sum[w][t][8];
+          any = true;
+        }
+      if (any) atomicAdd(sum9(g2d, q0 + s_gid[t], n_entries), sum);
     }
   }
 }
@@ -358,10 +462,17 @@ preprocess_backward_kernel(const PreParams *__restrict__ pp, int n, const float 
   float *dsh = s_dsh + threadIdx.x * SS;
 
   for (int e = 0; e < p.n_eyes; ++e) {
-    if (rec[((size_t)e * n + i) * kRec + 11] == 0.0f) continue;   // culled for this eye
-    const float *g = g2d + ((size_t)e * n + i) * kG2;
-    const float gu = g[0], gv = g[1], gca = g[2], gcb = g[3], gcc = g[4], gop = g[5];
-    const float gr[3] = {g[6], g[7], g[8]};
+    const size_t q = (size_t)e * n + i;
+    if (__ldg(rec + q * kRec + 11) == 0.0f) continue;   // culled for this eye
+    const float4 r0 = __ldg(reinterpret_cast<const float4 *>(rec + q * kRec));
+    const float conic_c = __ldg(rec + q * kRec + 4);
+    const float4 s0 = __ldg(reinterpret_cast<const float4 *>(g2d + 8 * q));
+    const float4 s1 = __ldg(reinterpret_cast<const float4 *>(g2d + 8 * q) + 1);
+    // power = -0.5 (a dx^2 + c dy^2) - b dx dy with dx = u - x, dy = v - y: the sums of dL/dpower
+    // times dx, dy, dx^2, dx dy, dy^2 (composite_backward) give the mean's and the conic's gradients
+    const float gu = -(r0.z * s0.x + r0.w * s0.y), gv = -(conic_c * s0.y + r0.w * s0.x);
+    const float gca = -0.5f * s0.z, gcb = -s0.w, gcc = -0.5f * s1.x, gop = s1.y;
+    const float gr[3] = {s1.z, s1.w, __ldg(g2d + 8 * (size_t)p.n_eyes * n + q)};
     const CamParams &c = p.cam[e];
     const float *W = c.R;
     const float tx = W[0] * mx + W[1] * my + W[2] * mz + c.t[0];
@@ -533,9 +644,15 @@ cudaError_t launch_backward(const BackwardParams &bp, const PreParams *pre_dev, 
   if (bp.n <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(g2d, 0, sizeof(float) * backward_g2d_floats(bp.n_eyes, bp.n), s);
   if (e != cudaSuccess) return e;
-  const int quads = (bp.tile / kTile) * (bp.tile / kTile);
-  composite_backward_kernel<<<bp.n_eyes * bp.n_tiles * quads, kThreads, 0, s>>>(
-      bp, rec, ranges, kept, vals, levels, t_final, n_contrib, dl_drgb, g2d);
+  const int quads = bp.n_eyes * bp.n_tiles * (bp.tile / kTile) * (bp.tile / kTile);
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (quads <= kSplitQuadsPerSm * sms)
+    composite_backward_kernel<1><<<2 * quads, kThreads, 0, s>>>(bp, rec, ranges, kept, vals, levels, t_final,
+                                                                n_contrib, dl_drgb, g2d);
+  else
+    composite_backward_kernel<2><<<quads, kThreads, 0, s>>>(bp, rec, ranges, kept, vals, levels, t_final, n_contrib,
+                                                            dl_drgb, g2d);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int blocks = (bp.n + kPreBwdThreads - 1) / kPreBwdThreads;
