@@ -10,9 +10,8 @@
 // scalar D carries it:  dL/dalpha_i = T_i (c_i . g - D_i),  D_{i-1} = alpha_i c_i . g +
 // (1 - alpha_i) D_i.  Alpha is recomputed exactly as the forward computed it (shared
 // helpers, explicitly rounded), so every skip / accept decision is the forward's.  Nine sums over
-// the pixels -- w g (three), dL/dopacity, and with p = dL/dpower those of p dx, p dy, p dx^2,
-// p dx dy, p dy^2 -- go to a per-(eye, Gaussian) buffer; what is linear in the conic is left to
-// preprocess_backward.  A foveated render's inherited pixels pass their gradient to the top-left
+// the pixels -- w g (three), dL/dopacity, and with p = dL/dpower and the falloff's A, B, C those of
+// p (2 A dx + B dy), p (2 C dy + B dx), p dx^2, p dx dy, p dy^2 -- go to a per-(eye, Gaussian) buffer.  A foveated render's inherited pixels pass their gradient to the top-left
 // pixel of their block.
 //
 // preprocess_backward: one thread per Gaussian, summing the eyes: conic -> 2-D covariance
@@ -21,6 +20,7 @@
 // through the sigmoid; colour -> SH coefficients and, through the view direction, mean.
 #include "blend.cuh"
 #include "common.cuh"
+#include "stage.cuh"
 
 namespace a3fr {
 namespace {
@@ -30,12 +30,14 @@ constexpr int kThreads = 128;            // four warps
 constexpr int kBatch = 128;              // Gaussians staged per batch
 constexpr int kG2 = 9;                   // sums per (eye, Gaussian): eight side by side, the ninth apart
 constexpr int kPreBwdThreads = 128;
+constexpr int kPreBwdCtas = 6;           // CTAs per SM
 // Quadrants are split in halves up to this many per SM, as the forward's 16-pixel tiles are: split /
-// not, 825 quadrants 102 / 145 us, 4,096 quadrants 160 / 146 us (ncu).
+// not, 825 quadrants 102 / 145 us, 4,096 quadrants 160 / 146 us (ncu, before the first-order sums
+// were formed per pixel).
 constexpr int kSplitQuadsPerSm = 16;
 
-// Where the sums of (eye, Gaussian) entry q of n_entries lie: [n_entries][8] -- p dx, p dy, p dx^2,
-// p dx dy, p dy^2, dopacity, dr, dg (one 32-byte sector) -- then [n_entries] db.
+// Where the sums of (eye, Gaussian) entry q of n_entries lie: [n_entries][8] -- the five of p,
+// dopacity, dr, dg (one 32-byte sector) -- then [n_entries] db.
 __device__ __forceinline__ float *sums8(float *g2d, size_t q) { return g2d + 8 * q; }
 __device__ __forceinline__ float *sum9(float *g2d, size_t q, size_t n_entries) { return g2d + 8 * n_entries + q; }
 
@@ -47,7 +49,7 @@ __device__ __forceinline__ float *sum9(float *g2d, size_t q, size_t n_entries) {
 // one reduction per value, Gaussian and quadrant.
 // Bound by issue, and by the longest list's chain on small images.  1M Gaussians at 1024 x 1024 (ncu):
 // 281 us with every warp (16 x 2 pixels) walking the whole list and adding its own nine sums to
-// memory, 146 us now; 50k at 517 x 389: 247, 102 us.
+// memory, 154 us now; 50k at 517 x 389: 247, 106 us.
 template <int Q>
 __global__ void __launch_bounds__(kThreads, 6)
 composite_backward_kernel(BackwardParams p, const float *__restrict__ rec, const uint2 *__restrict__ ranges,
@@ -212,8 +214,12 @@ composite_backward_kernel(BackwardParams p, const float *__restrict__ rec, const
           f2_unpack(f2_fma(a2, cdot, f2_mul(om, D2)), D[0], D[Q - 1]);
           const f32x2 dpow = f2_mul(dal, f2_pack(free0 ? ar0 : 0.0f, free1 ? ar1 : 0.0f));
           const f32x2 px2 = f2_mul(dpow, dx), py2 = f2_mul(dpow, dy);
-          v[u][0] = f2_sum(px2);
-          v[u][1] = f2_sum(py2);
+          // 2 A dx + B dy and 2 C dy + B dx per pixel, before the sum: in an elongated Gaussian the
+          // two terms nearly cancel
+          const f32x2 bx = f2_pack(geo.w, geo.w);
+          const float A2 = geo.z + geo.z, C2 = crg.x + crg.x;
+          v[u][0] = f2_sum(f2_mul(dpow, f2_fma(f2_pack(A2, A2), dx, f2_mul(bx, dy))));
+          v[u][1] = f2_sum(f2_mul(dpow, f2_fma(f2_pack(C2, C2), dy, f2_mul(bx, dx))));
           v[u][2] = f2_sum(f2_mul(px2, dx));
           v[u][3] = f2_sum(f2_mul(px2, dy));
           v[u][4] = f2_sum(f2_mul(py2, dy));
@@ -237,11 +243,11 @@ composite_backward_kernel(BackwardParams p, const float *__restrict__ rec, const
           const float dal = T[0] * (cdot - D[0]);
           D[0] = a * cdot + om * D[0];
           const float dpow = dal * (open ? araw : 0.0f);
-          v[u][0] = dpow * dx;
-          v[u][1] = dpow * dy;
-          v[u][2] = v[u][0] * dx;
-          v[u][3] = v[u][0] * dy;
-          v[u][4] = v[u][1] * dy;
+          v[u][0] = dpow * (2.0f * geo.z * dx + geo.w * dy);
+          v[u][1] = dpow * (2.0f * crg.x * dy + geo.w * dx);
+          v[u][2] = dpow * dx * dx;
+          v[u][3] = dpow * dx * dy;
+          v[u][4] = dpow * dy * dy;
           v[u][5] = dal * (open ? G : 0.0f);
           v[u][6] = w * g[0][0];
           v[u][7] = w * g[0][1];
@@ -382,20 +388,36 @@ __device__ __forceinline__ void sh_basis_vjp(const ShConsts &c, float x, float y
   }
 }
 
-// Shared-memory row stride (floats) of a block's SH coefficients and their gradients: the
-// 3K coefficients rounded up to an odd count, so the threads of a warp, reading the same
-// coefficient of consecutive rows, hit distinct banks.
-template <int K> constexpr int sh_stride() { return (3 * K) % 2 ? 3 * K : 3 * K + 1; }
-template <int K> constexpr size_t backward_smem_bytes() {
-  return 2 * sizeof(float) * (size_t)kPreBwdThreads * sh_stride<K>();
+// Calls f(index, element) for the 3K elements of thread t's SH row in shared memory (the layouts of
+// stage.cuh), four to a 16-byte access where rows are whole chunks; kStore writes them back.
+template <int K, bool kStore, typename F>
+__device__ __forceinline__ void each_sh(float *rows, int t, F f) {
+  if constexpr (sh_chunked<K>()) {
+    float4 *row4 = reinterpret_cast<float4 *>(rows + t * 3 * K);
+#pragma unroll
+    for (int m = 0; m < 3 * K / 4; ++m) {
+      const float4 v = row4[sh_swz<K>(m, t)];
+      float e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) f(4 * m + j, e[j]);
+      if (kStore) row4[sh_swz<K>(m, t)] = make_float4(e[0], e[1], e[2], e[3]);
+    }
+  } else {
+    float *row = rows + t * sh_stride<K>();
+#pragma unroll
+    for (int j = 0; j < 3 * K; ++j) f(j, row[j]);
+  }
 }
 
-// One thread per Gaussian.  The block's SH coefficients are copied into shared memory with
-// coalesced loads and their gradients accumulated there, then written back coalesced (read
-// and accumulated per thread in global memory, the 48-float rows made every access a
-// separate sector).
+// One thread per Gaussian.  The block's SH rows are copied into shared memory asynchronously while
+// the threads load the rest; a row is read for every eye, then overwritten by its gradient (the
+// eyes' directions and colour gradients are kept, their bases evaluated again), and the rows are
+// written back coalesced.
+// Bound by memory: 1M Gaussians, SH degree 3 (556 MB) 125 us under ncu; 196 us with the rows and
+// their gradients in separate arrays copied by plain loads (50 KB and 127 registers: 16 warps per SM,
+// waiting on memory).
 template <int K>
-__global__ void __launch_bounds__(kPreBwdThreads)
+__global__ void __launch_bounds__(kPreBwdThreads, kPreBwdCtas)
 preprocess_backward_kernel(const PreParams *__restrict__ pp, int n, const float *__restrict__ means,
                            const float *__restrict__ log_scales, const float *__restrict__ quats,
                            const float *__restrict__ opacity_logits, const float *__restrict__ sh,
@@ -403,28 +425,21 @@ preprocess_backward_kernel(const PreParams *__restrict__ pp, int n, const float 
                            float *__restrict__ d_means, float *__restrict__ d_log_scales,
                            float *__restrict__ d_quats, float *__restrict__ d_logits,
                            float *__restrict__ d_sh) {
-  constexpr int SS = sh_stride<K>();
   constexpr int ROW = 3 * K;
   __shared__ PreParams s_p;
-  extern __shared__ float s_sh_dyn[];
-  float *s_coef = s_sh_dyn;                          // [kPreBwdThreads][SS]
-  float *s_dsh = s_sh_dyn + kPreBwdThreads * SS;     // [kPreBwdThreads][SS]
+  __shared__ __align__(16) float s_sh[kPreBwdThreads * sh_stride<K>()];
   static_assert(sizeof(PreParams) % 4 == 0 && sizeof(PreParams) / 4 <= kPreBwdThreads, "PreParams copy");
-  if (threadIdx.x < sizeof(PreParams) / 4)
-    reinterpret_cast<uint32_t *>(&s_p)[threadIdx.x] = reinterpret_cast<const uint32_t *>(pp)[threadIdx.x];
   const int i0 = blockIdx.x * kPreBwdThreads;
   const int rows = min(kPreBwdThreads, n - i0);
-  {
-    const float *src = sh + (size_t)ROW * i0;
-    for (int f = threadIdx.x; f < rows * ROW; f += kPreBwdThreads) {
-      const int r = f / ROW, c = f - r * ROW;
-      s_coef[r * SS + c] = src[f];
-      s_dsh[r * SS + c] = 0.0f;
-    }
-  }
+  const int t = threadIdx.x;
+  if constexpr (sh_chunked<K>()) stage_sh_async<K>(s_sh, sh + (size_t)ROW * i0, rows);
+  if (t < sizeof(PreParams) / 4)
+    reinterpret_cast<uint32_t *>(&s_p)[t] = reinterpret_cast<const uint32_t *>(pp)[t];
+  if constexpr (!sh_chunked<K>()) stage(s_sh, sh + (size_t)ROW * i0, rows * ROW, ROW, sh_stride<K>());
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   const PreParams &p = s_p;
-  const int i = i0 + threadIdx.x;
+  const int i = i0 + t;
   if (i < n) {
 
   const float mx = means[3 * i], my = means[3 * i + 1], mz = means[3 * i + 2];
@@ -454,23 +469,24 @@ preprocess_backward_kernel(const PreParams *__restrict__ pp, int n, const float 
     for (int k = 0; k < 3; ++k)
       S[j][k] = R[j][0] * s2[0] * R[k][0] + R[j][1] * s2[1] * R[k][1] + R[j][2] * s2[2] * R[k][2];
   const float opacity = 1.0f / (1.0f + expf(-opacity_logits[i]));
-  const float *coef = s_coef + threadIdx.x * SS;
 
   float dmu[3] = {0.f, 0.f, 0.f};
   float dS[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
   float dlogit = 0.0f;
-  float *dsh = s_dsh + threadIdx.x * SS;
+  float dir[kMaxEyes][3], gcol[kMaxEyes][3];   // per eye: direction, gradient of the colour
 
-  for (int e = 0; e < p.n_eyes; ++e) {
+#pragma unroll
+  for (int e = 0; e < kMaxEyes; ++e) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) dir[e][k] = gcol[e][k] = 0.0f;
+    if (e >= p.n_eyes) continue;
     const size_t q = (size_t)e * n + i;
     if (__ldg(rec + q * kRec + 11) == 0.0f) continue;   // culled for this eye
-    const float4 r0 = __ldg(reinterpret_cast<const float4 *>(rec + q * kRec));
-    const float conic_c = __ldg(rec + q * kRec + 4);
     const float4 s0 = __ldg(reinterpret_cast<const float4 *>(g2d + 8 * q));
     const float4 s1 = __ldg(reinterpret_cast<const float4 *>(g2d + 8 * q) + 1);
-    // power = -0.5 (a dx^2 + c dy^2) - b dx dy with dx = u - x, dy = v - y: the sums of dL/dpower
-    // times dx, dy, dx^2, dx dy, dy^2 (composite_backward) give the mean's and the conic's gradients
-    const float gu = -(r0.z * s0.x + r0.w * s0.y), gv = -(conic_c * s0.y + r0.w * s0.x);
+    // power = -0.5 (a dx^2 + c dy^2) - b dx dy with dx = u - x, dy = v - y; in base 2, as
+    // composite_backward sums it, A = -0.5 log2(e) a, B = -log2(e) b, C = -0.5 log2(e) c
+    const float gu = s0.x * (1.0f / kLog2e), gv = s0.y * (1.0f / kLog2e);
     const float gca = -0.5f * s0.z, gcb = -s0.w, gcc = -0.5f * s1.x, gop = s1.y;
     const float gr[3] = {s1.z, s1.w, __ldg(g2d + 8 * (size_t)p.n_eyes * n + q)};
     const CamParams &c = p.cam[e];
@@ -563,23 +579,21 @@ preprocess_backward_kernel(const PreParams *__restrict__ pp, int n, const float 
     const float ddx = mx - C[0], ddy = my - C[1], ddz = mz - C[2];
     const float dn = sqrtf(ddx * ddx + ddy * ddy + ddz * ddz);
     const float x = ddx / dn, y = ddy / dn, z = ddz / dn;
-    float Y[K];
-    sh_basis_eval<K>(p.shc, x, y, z, Y);
-    float gch[3];
-#pragma unroll
-    for (int ch = 0; ch < 3; ++ch) {
-      float acc = 0.5f;
-#pragma unroll
-      for (int k = 0; k < K; ++k) acc += Y[k] * coef[3 * k + ch];
-      gch[ch] = acc > 0.0f ? gr[ch] : 0.0f;   // max(0, .) passes gradient where positive
+    dir[e][0] = x;
+    dir[e][1] = y;
+    dir[e][2] = z;
+    float acc[3] = {0.5f, 0.5f, 0.5f};
+    {
+      float Y[K];
+      sh_basis_eval<K>(p.shc, x, y, z, Y);
+      each_sh<K, false>(s_sh, t, [&](int f, float &c) { acc[f % 3] += Y[f / 3] * c; });
     }
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) gcol[e][ch] = acc[ch] > 0.0f ? gr[ch] : 0.0f;   // max(0, .): where positive
     float wk[K];
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      wk[k] = coef[3 * k] * gch[0] + coef[3 * k + 1] * gch[1] + coef[3 * k + 2] * gch[2];
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) dsh[3 * k + ch] += Y[k] * gch[ch];
-    }
+    for (int k = 0; k < K; ++k) wk[k] = 0.0f;
+    each_sh<K, false>(s_sh, t, [&](int f, float &c) { wk[f / 3] += c * gcol[e][f % 3]; });
     float gx, gy, gz;
     sh_basis_vjp<K>(p.shc, x, y, z, wk, gx, gy, gz);
     const float dot = x * gx + y * gy + z * gz;
@@ -621,12 +635,32 @@ preprocess_backward_kernel(const PreParams *__restrict__ pp, int n, const float 
   d_means[3 * i + 1] = dmu[1];
   d_means[3 * i + 2] = dmu[2];
   d_logits[i] = dlogit;
+  // the SH gradient in place of the row
+  {
+    float Y[K];
+    sh_basis_eval<K>(p.shc, dir[0][0], dir[0][1], dir[0][2], Y);
+    each_sh<K, true>(s_sh, t, [&](int f, float &c) { c = Y[f / 3] * gcol[0][f % 3]; });
+    if (p.n_eyes > 1) {
+      sh_basis_eval<K>(p.shc, dir[1][0], dir[1][1], dir[1][2], Y);
+      each_sh<K, true>(s_sh, t, [&](int f, float &c) { c += Y[f / 3] * gcol[1][f % 3]; });
+    }
+  }
   }
   __syncthreads();
   float *dst = d_sh + (size_t)ROW * i0;
-  for (int f = threadIdx.x; f < rows * ROW; f += kPreBwdThreads) {
-    const int r = f / ROW, c = f - r * ROW;
-    dst[f] = s_dsh[r * SS + c];
+  if constexpr (sh_chunked<K>()) {
+    if ((reinterpret_cast<uintptr_t>(d_sh) & 15u) == 0u) {
+      for (int c = t; c < rows * (ROW / 4); c += kPreBwdThreads) {
+        const int r = c / (ROW / 4), m = c - r * (ROW / 4);
+        reinterpret_cast<float4 *>(dst)[c] = reinterpret_cast<const float4 *>(s_sh + r * ROW)[sh_swz<K>(m, r)];
+      }
+      return;
+    }
+  }
+  for (int f = t; f < rows * ROW; f += kPreBwdThreads) {
+    const int r = f / ROW, c = f % ROW;
+    if constexpr (sh_chunked<K>()) dst[f] = s_sh[r * ROW + 4 * sh_swz<K>(c >> 2, r) + (c & 3)];
+    else dst[f] = s_sh[r * sh_stride<K>() + c];
   }
 }
 
@@ -656,20 +690,16 @@ cudaError_t launch_backward(const BackwardParams &bp, const PreParams *pre_dev, 
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int blocks = (bp.n + kPreBwdThreads - 1) / kPreBwdThreads;
-  auto go = [&](auto kern, size_t smem) -> cudaError_t {
-    // per device: the attribute lives in each device's context
-    cudaError_t e2 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e2 != cudaSuccess) return e2;
-    kern<<<blocks, kPreBwdThreads, smem, s>>>(pre_dev, bp.n, means, log_scales, quats, opacity_logits,
-                                               sh, rec, g2d, d_means, d_log_scales, d_quats, d_logits,
-                                               d_sh);
+  auto go = [&](auto kern) -> cudaError_t {
+    kern<<<blocks, kPreBwdThreads, 0, s>>>(pre_dev, bp.n, means, log_scales, quats, opacity_logits, sh, rec, g2d,
+                                           d_means, d_log_scales, d_quats, d_logits, d_sh);
     return cudaGetLastError();
   };
   switch (sh_degree) {
-    case 0: return go(preprocess_backward_kernel<1>, backward_smem_bytes<1>());
-    case 1: return go(preprocess_backward_kernel<4>, backward_smem_bytes<4>());
-    case 2: return go(preprocess_backward_kernel<9>, backward_smem_bytes<9>());
-    default: return go(preprocess_backward_kernel<16>, backward_smem_bytes<16>());
+    case 0: return go(preprocess_backward_kernel<1>);
+    case 1: return go(preprocess_backward_kernel<4>);
+    case 2: return go(preprocess_backward_kernel<9>);
+    default: return go(preprocess_backward_kernel<16>);
   }
 }
 
