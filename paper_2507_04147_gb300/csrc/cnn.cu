@@ -95,43 +95,7 @@ struct ConvDims {
   int B, H, W;
 };
 
-enum : int { kEpiBias = 1, kEpiRelu = 2, kEpiResid = 4, kEpiMask = 8, kEpiF32 = 16 };
-
-// Halo rows x cols of 8-channel groups around the tile whose top-left output pixel is (y0, x0).
-template <int CG>
-__device__ __forceinline__ void load_halo(uint8_t *hs, const __nv_bfloat16 *__restrict__ X, int b,
-                                          int y0, int x0, int rows, int cols, int H, int W) {
-  const int total = rows * cols * CG;
-  for (int i = threadIdx.x; i < total; i += blockDim.x) {
-    const int cg = i % CG, rc = i / CG;
-    const int c = rc % cols, r = rc / cols;
-    const int y = y0 - 1 + r, x = x0 - 1 + c;
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (y >= 0 && y < H && x >= 0 && x < W)
-      v = __ldg(reinterpret_cast<const uint4 *>(X + (((size_t)b * H + y) * W + x) * (CG * 8)) + cg);
-    *reinterpret_cast<uint4 *>(hs + ((size_t)(cg * rows + r) * cols + c) * 16) = v;
-  }
-}
-
-// The same halo with asynchronous 16-byte copies (zero-filled outside the image); the caller
-// waits with cp_async_wait_all() before the data is used.
-template <int CG>
-__device__ __forceinline__ void load_halo_async(uint8_t *hs, const __nv_bfloat16 *__restrict__ X, int b,
-                                                int y0, int x0, int rows, int cols, int H, int W) {
-  const int total = rows * cols * CG;
-  for (int i = threadIdx.x; i < total; i += blockDim.x) {
-    const int cg = i % CG, rc = i / CG;
-    const int c = rc % cols, r = rc / cols;
-    const int y = y0 - 1 + r, x = x0 - 1 + c;
-    const bool in = y >= 0 && y < H && x >= 0 && x < W;
-    const __nv_bfloat16 *src = in ? X + (((size_t)b * H + y) * W + x) * (CG * 8) + cg * 8 : X;
-    const uint32_t dst = tc::smem_u32(hs + ((size_t)(cg * rows + r) * cols + c) * 16);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0)
-                 : "memory");
-  }
-  asm volatile("cp.async.commit_group;" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+enum : int { kEpiBias = 1, kEpiRelu = 2, kEpiResid = 4, kEpiMask = 8, kEpiF32 = 16, kBiasRelu = kEpiBias | kEpiRelu };
 
 // The image side of the learned fill, for the two convolutions that touch it when the fill
 // runs fused: the first reads its input straight from the render (kSrcImage), the last
@@ -146,18 +110,21 @@ struct FillIO {
 enum : int { kSrcTensor = 0, kSrcImage = 1 };
 enum : int { kDstTensor = 0, kDstCompose = 1 };
 
-// The 16 input channels of block (y2, x2): r, g, b of its top-left pixel and depth / 8 in
-// BF16, then zeros (the first eight as one 16-byte group; the second group is all zero).
-__device__ __forceinline__ uint4 block_input(const float *__restrict__ img, const float *__restrict__ depth,
-                                             int b, int H, int W, int y2, int x2) {
-  const size_t src = ((size_t)b * H + 2 * y2) * W + 2 * x2;
+// The first eight of a block's 16 input channels: r, g, b of its top-left pixel and depth / 8 in
+// BF16, then zeros (as are the other eight).
+__device__ __forceinline__ uint4 block_operand(float4 v) {
   uint4 lo;
   __nv_bfloat162 *l2 = reinterpret_cast<__nv_bfloat162 *>(&lo);
-  l2[0] = __floats2bfloat162_rn(img[3 * src], img[3 * src + 1]);
-  l2[1] = __floats2bfloat162_rn(img[3 * src + 2], depth[src] * 0.125f);
+  l2[0] = __floats2bfloat162_rn(v.x, v.y);
+  l2[1] = __floats2bfloat162_rn(v.z, v.w * 0.125f);
   l2[2] = __floats2bfloat162_rn(0.0f, 0.0f);
   l2[3] = l2[2];
   return lo;
+}
+__device__ __forceinline__ uint4 block_input(const float *__restrict__ img, const float *__restrict__ depth,
+                                             int b, int H, int W, int y2, int x2) {
+  const size_t src = ((size_t)b * H + 2 * y2) * W + 2 * x2;
+  return block_operand(make_float4(img[3 * src], img[3 * src + 1], img[3 * src + 2], depth[src]));
 }
 
 // Final image of a foveated render at block (y2, x2) from its 12 residuals res[c][2 dy + dx]:
@@ -197,214 +164,340 @@ __device__ __forceinline__ void compose_block(float *__restrict__ img, int b, in
   if (lv <= 1) put(1, 1, bd);   // bottom-right: label 2, rendered from level 2
 }
 
-template <int CIN, int COUT>
-constexpr int conv_smem_bytes() {
-  return 2 * (CIN / 8) * (kConvTH + 2) * (kConvTW + 2) * 16 + 9 * (CIN / 8) * COUT * 16;
+// Lane j of four has a[0..4): afterwards a[i] is what lane i had as a[j].
+__device__ __forceinline__ void transpose4(uint4 (&a)[4]) {
+  const bool b0 = threadIdx.x & 1, b1 = threadIdx.x & 2;
+  auto swap = [](uint4 &p, uint4 &q, bool up, int mask) {   // up: p is what the partner wants, else q
+    const uint4 s = up ? p : q;
+    uint4 r;
+    r.x = __shfl_xor_sync(0xffffffffu, s.x, mask);
+    r.y = __shfl_xor_sync(0xffffffffu, s.y, mask);
+    r.z = __shfl_xor_sync(0xffffffffu, s.z, mask);
+    r.w = __shfl_xor_sync(0xffffffffu, s.w, mask);
+    if (up) p = r;
+    else q = r;
+  };
+  swap(a[0], a[1], b0, 1);
+  swap(a[2], a[3], b0, 1);
+  swap(a[0], a[2], b1, 2);
+  swap(a[1], a[3], b1, 2);
 }
 
-// Persistent over 8 x 16 output tiles (128 threads: one per output pixel in the epilogue).  A
-// CTA loads the layer's packed weights once, then walks tiles blockIdx.x, + gridDim.x, ...
-// with a two-deep pipeline: two halo buffers in shared memory and two 32-column accumulators
-// in tensor memory, so the halo of tile k+1 loads while tile k's MMAs run, and tile k's
-// epilogue (tensor-memory read, bias, ReLU, residual, mask, store) runs while tile k+1's MMAs
-// do.  One thread issues the 9 x (CIN/16) MMAs of a tile and commits them to the mbarrier;
-// tile k completes phase k.
+// The tiles blockIdx.x, + gridDim.x, + 2 gridDim.x ... of B x tiles_y x tiles_x, by additions.
+struct TileWalk {
+  int tx, ty, b;
+  __device__ __forceinline__ TileWalk(int tiles_x, int tiles_y) : nx(tiles_x), ny(tiles_y) {
+    split((int)blockIdx.x, tx, ty, b);
+    split((int)gridDim.x, dx, dy, db);
+  }
+  __device__ __forceinline__ void next() {
+    tx += dx;
+    ty += dy;
+    b += db;
+    if (tx >= nx) {
+      tx -= nx;
+      ++ty;
+    }
+    if (ty >= ny) {
+      ty -= ny;
+      ++b;
+    }
+  }
+
+ private:
+  int nx, ny, dx, dy, db;
+  __device__ __forceinline__ void split(int i, int &x, int &y, int &z) const {
+    x = i % nx;
+    y = i / nx % ny;
+    z = i / nx / ny;
+  }
+};
+
+// Persistent over 8 x 16 output tiles, one CTA per SM, warp-specialised: eight warps copy input
+// halos into a ring of stages; two warps issue the 9 x (CIN/16) MMAs of a tile, in turn, into the stage's own
+// 32-column accumulator, so that one commit frees the halo and hands over the accumulator; two groups
+// of four warps take the tiles in turn for the epilogue (tensor-memory read, bias, ReLU, residual,
+// mask, store; one output pixel a thread), each loading its next tile's residual and mask before the
+// current one's accumulator is complete.  What the epilogue does is a template parameter.
 //
-// kSrcImage (16 input channels): the halo is formed from the render (block_input) instead of
-// copied from a tensor -- its loads issued before tile k's epilogue, stored to shared memory
-// after it.  kDstCompose (16 output channels): the epilogue composes the block's skipped
-// pixels into the image (compose_block) instead of storing the residuals.
-template <int CIN, int COUT, int SRC = kSrcTensor, int DST = kDstTensor>
-__global__ void __launch_bounds__(128)
+// kSrcImage (16 input channels): the halo is formed from the render (block_operand) instead of copied
+// from a tensor.  kDstCompose (16 output channels): the epilogue composes the block's skipped pixels
+// into the image (compose_block) instead of storing the residuals.
+//
+// What the parts do for a tile is short (18 MMAs of about 32 clocks, 11 KB loaded, 8 KB stored), so
+// the time goes to latencies and the rings' depth decides: with residual on 2 x 1104 x 1032 pixels
+// (32 -> 32, 438 MB, 65 us at the measured copy rate) 92 us under ncu with 12 stages, 108 us with 6;
+// 131 us with one MMA warp and copies straight to shared memory, 140 us with five CTAs of 128 threads
+// per SM that each loaded, multiplied and stored in turn.  Without it 102 -> 80 us; 16 x 128 x 128
+// pixels 22 -> 15 us.  MMAs of several tiles interleaved in one issue stream: no faster.
+constexpr int kConvStages = 12;                    // even: see the parities below; 32 accumulator columns each
+constexpr int kConvThreads = 2 * 128 + 2 * 128 + 2 * 32;   // epilogue groups, copying groups, MMA warps
+constexpr int kConvHR = kConvTH + 2, kConvHC = kConvTW + 2;
+// one plane of 8 channels; the padding puts a pixel's groups in different banks (CIN 32)
+constexpr int kConvPlane = kConvHR * kConvHC * 16 + 96;
+
+template <int CIN, int COUT>
+constexpr int conv_smem_bytes() { return kConvStages * (CIN / 8) * kConvPlane + 9 * (CIN / 8) * COUT * 16; }
+
+template <int CIN, int COUT, int FLAGS, int SRC, int DST>
+__global__ void __launch_bounds__(kConvThreads, 1)
 conv3x3_tc_kernel(ConvDims d, const __nv_bfloat16 *__restrict__ X, const uint4 *__restrict__ Wpk,
                   const float *__restrict__ bias, const __nv_bfloat16 *__restrict__ R,
-                  const __nv_bfloat16 *__restrict__ Mk, void *__restrict__ Y, int flags,
-                  uint32_t *__restrict__ status, FillIO io) {
+                  const __nv_bfloat16 *__restrict__ Mk, void *__restrict__ Y, uint32_t *__restrict__ status,
+                  FillIO io) {
   static_assert(SRC == kSrcTensor || CIN == 16, "the image input has 16 channels");
   static_assert(DST == kDstTensor || COUT == 16, "the composed residuals have 16 channels");
-  constexpr int CG = CIN / 8, HR = kConvTH + 2, HC = kConvTW + 2;
-  constexpr int HALO = CG * HR * HC * 16, WBYTES = 9 * CG * COUT * 16;
-  constexpr int kGPer = (HR * HC + 127) / 128;   // halo pixels per thread (image input)
+  constexpr int CG = CIN / 8, HR = kConvHR, HC = kConvHC, S = kConvStages;
+  constexpr int HALO = CG * kConvPlane, WBYTES = 9 * CG * COUT * 16;
   extern __shared__ __align__(1024) uint8_t smem[];
-  uint8_t *const ws = smem + 2 * HALO;
+  uint8_t *const ws = smem + S * HALO;
   __shared__ uint32_t s_tmem;
-  __shared__ __align__(8) uint64_t s_bar;
-  __shared__ float s_bias[32];
+  __shared__ __align__(8) uint64_t s_full[S], s_done[S], s_free[S];   // halo landed, MMAs done, accumulator read
+  __shared__ __align__(16) float s_bias[32];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  if (t < COUT) s_bias[t] = (flags & kEpiBias) ? bias[t] : 0.0f;
   const int tiles_x = (d.W + kConvTW - 1) / kConvTW, tiles_y = (d.H + kConvTH - 1) / kConvTH;
   const int n_tiles = d.B * tiles_x * tiles_y;
-  const int my_n = (int)blockIdx.x < n_tiles ? (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-  auto origin = [&](int k, int &b, int &y0, int &x0) {
-    const int tt = (int)blockIdx.x + k * (int)gridDim.x;
-    x0 = (tt % tiles_x) * kConvTW;
-    const int r = tt / tiles_x;
-    y0 = (r % tiles_y) * kConvTH;
-    b = r / tiles_y;
-  };
-  // image input: the halo pixels of a tile, loaded into registers, then stored as BF16 groups
-  // (the second 8-channel group stays zero: it is cleared once here)
-  uint4 gv[kGPer];
-  auto gather_load = [&](int k) {
-    int b, y0, x0;
-    origin(k, b, y0, x0);
-#pragma unroll
-    for (int j = 0; j < kGPer; ++j) {
-      const int q = t + 128 * j, r = q / HC, c = q - r * HC;
-      const int y = y0 - 1 + r, x = x0 - 1 + c;
-      gv[j] = make_uint4(0u, 0u, 0u, 0u);
-      if (q < HR * HC && y >= 0 && y < d.H && x >= 0 && x < d.W)
-        gv[j] = block_input(io.img, io.depth, b, io.H, io.W, y, x);
+  const int my_n = (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // grid <= n_tiles
+  if (warp == 16) tc::tmem_alloc(&s_tmem, 512);
+  if (t == 0) {
+    for (int k = 0; k < S; ++k) {
+      tc::mbar_init(&s_full[k], 4);
+      tc::mbar_init(&s_done[k], 1);
+      tc::mbar_init(&s_free[k], 4);
     }
-  };
-  auto gather_store = [&](uint8_t *hs) {
-#pragma unroll
-    for (int j = 0; j < kGPer; ++j) {
-      const int q = t + 128 * j;
-      if (q < HR * HC) *reinterpret_cast<uint4 *>(hs + (size_t)q * 16) = gv[j];
-    }
-  };
-  if (warp == 0) tc::tmem_alloc(&s_tmem, 64);
-  for (int i = t; i < WBYTES / 16; i += 128) reinterpret_cast<uint4 *>(ws)[i] = __ldg(Wpk + i);
-  if constexpr (SRC == kSrcImage) {
-    for (int i = t; i < 2 * HR * HC; i += 128) {   // group 1 of both halo buffers
-      const int buf = i / (HR * HC), q = i - buf * (HR * HC);
-      *reinterpret_cast<uint4 *>(smem + buf * HALO + (size_t)(HR * HC + q) * 16) = make_uint4(0u, 0u, 0u, 0u);
-    }
-    if (my_n > 0) {
-      gather_load(0);
-      gather_store(smem);
-    }
-  } else if (my_n > 0) {
-    int b, y0, x0;
-    origin(0, b, y0, x0);
-    load_halo_async<CG>(smem, X, b, y0, x0, HR, HC, d.H, d.W);
   }
-  cp_async_wait_all();
+  pdl_begin();
+  for (int i = t; i < WBYTES / 16; i += kConvThreads) reinterpret_cast<uint4 *>(ws)[i] = __ldg(Wpk + i);
+  if (t < COUT) s_bias[t] = (FLAGS & kEpiBias) ? bias[t] : 0.0f;
+  if constexpr (SRC == kSrcImage) {
+    for (int i = t; i < S * HR * HC; i += kConvThreads) {   // the second input group is zero
+      const int st = i / (HR * HC), q = i - st * (HR * HC);
+      *reinterpret_cast<uint4 *>(smem + st * HALO + kConvPlane + q * 16) = make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
   tc::fence_proxy_async();
-  if (t == 0) tc::mbar_init(&s_bar, 1);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = s_tmem;
-  const uint32_t idesc = tc::idesc_bf16_f32(128, COUT);
-  auto issue = [&](int k) {   // MMAs of tile k: halo buffer k & 1, accumulator columns 32 (k & 1)
-    const uint32_t h0 = tc::smem_u32(smem + (k & 1) * HALO), w0 = tc::smem_u32(ws);
-    const uint32_t dt = tmem + (uint32_t)((k & 1) * 32);
-    int n = 0;
-#pragma unroll 1
-    for (int tap = 0; tap < 9; ++tap) {
-      const int ky = tap / 3, kx = tap - 3 * ky;
+
+  if (warp >= 16) {
+    // two warps take the tiles in turn (one's waits overlap the other's issue); a whole warp runs the
+    // loop, so that descriptors stay in uniform registers, and one lane issues
+    const bool leader = tc::elect_one();
+    const uint32_t idesc = tc::idesc_bf16_f32(128, COUT), w0 = tc::smem_u32(ws), h00 = tc::smem_u32(smem);
+    for (int k = warp - 16, st = warp - 16, ph = 0; k < my_n; k += 2) {
+      bool ok = tc::mbar_wait(&s_full[st], ph);
+      if (k >= S) ok = tc::mbar_wait(&s_free[st], ph ^ 1) && ok;
+      if (!ok && leader) atomicOr(status, kStatusTimeout);
+      tc::fence_after_sync();
+      const uint32_t h0 = h00 + st * HALO;
 #pragma unroll
-      for (int cb = 0; cb < CIN / 16; ++cb) {
-        const uint64_t a = tc::smem_desc(h0 + (2 * cb) * (HR * HC * 16) + ky * (HC * 16) + kx * 16,
-                                         HR * HC * 16, HC * 16);
-        const uint64_t w = tc::smem_desc(w0 + tap * (CG * COUT * 16) + (2 * cb) * (COUT * 16), COUT * 16, 128);
-        tc::mma_bf16(dt, a, w, idesc, n > 0);
-        ++n;
+      for (int tap = 0; tap < 9; ++tap)
+#pragma unroll
+        for (int cb = 0; cb < CIN / 16; ++cb) {
+          const int ky = tap / 3, kx = tap - 3 * ky;
+          tc::mma_bf16_if(leader, tmem + 32 * st,
+                          tc::smem_desc(h0 + (2 * cb) * kConvPlane + ky * (HC * 16) + kx * 16, kConvPlane, HC * 16),
+                          tc::smem_desc(w0 + tap * (CG * COUT * 16) + (2 * cb) * (COUT * 16), COUT * 16, 128), idesc,
+                          tap > 0 || cb > 0);
+        }
+      if (leader) tc::mma_commit(&s_done[st]);
+      __syncwarp();
+      st += 2;   // S is even: a warp or group keeps its parity of stages
+      if (st >= S) {
+        st -= S;
+        ph ^= 1;
       }
     }
-    tc::mma_commit(&s_bar);
-  };
-  if (t == 0 && my_n > 0) issue(0);
-  if (my_n > 1) {   // buffer 1 is free: start tile 1's halo
-    if constexpr (SRC == kSrcImage) {
-      gather_load(1);
-      gather_store(smem + HALO);
-    } else {
-      int b, y0, x0;
-      origin(1, b, y0, x0);
-      load_halo_async<CG>(smem + HALO, X, b, y0, x0, HR, HC, d.H, d.W);
-    }
-  }
-  for (int k = 0; k < my_n; ++k) {
-    int b, y0, x0;
-    origin(k, b, y0, x0);
-    const int m = warp * 32 + lane;
-    const int y = y0 + m / kConvTW, x = x0 + (m % kConvTW);
-    const bool inside = y < d.H && x < d.W;
-    const size_t pix = inside ? ((size_t)b * d.H + y) * d.W + x : 0;
-    // the epilogue's residual input, loaded now so that its latency overlaps the waits for this
-    // tile's MMAs and the next halo
-    uint4 rv[COUT / 8];
-#pragma unroll
-    for (int g = 0; g < COUT / 8; ++g)
-      rv[g] = (inside && (flags & kEpiResid)) ? __ldg(reinterpret_cast<const uint4 *>(R + pix * COUT) + g)
-                                              : make_uint4(0u, 0u, 0u, 0u);
-    if (!tc::mbar_wait(&s_bar, (uint32_t)(k & 1)) && lane == 0) atomicOr(status, kStatusTimeout);
-    cp_async_wait_all();   // halo k + 1 has landed
-    tc::fence_proxy_async();
-    tc::fence_before_sync();
-    __syncthreads();   // halo k + 1 complete everywhere; every thread saw tile k complete
-    tc::fence_after_sync();
-    if (t == 0 && k + 1 < my_n) issue(k + 1);
-    if (k + 2 < my_n) {   // buffer k & 1 was read by tile k, which completed
+  } else if (warp >= 8) {
+    // Two groups of four warps take the tiles in turn, each with three register sets: a tile's loads
+    // are issued two of the group's tiles before they are stored, so that five tiles are in flight.  (Copies straight to shared memory would be one L2 request per 16
+    // bytes here -- neighbouring 16 bytes go to different planes -- and fetch every sector twice.)
+    const int group = (warp - 8) >> 2, lt = t & 127;
+    TileWalk at(tiles_x, tiles_y);
+    if (group == 1) at.next();
+    // image: two halo pixels a thread (180 of them), r g b depth; tensor: 120 threads, a column and
+    // channel group each, every (12 / CG)-th row
+    constexpr int RSTEP = 12 / CG, NV = SRC == kSrcImage ? 2 : HR / RSTEP;
+    const int lg = lt % CG, lc = (lt / CG) % HC, lrow = lt / (CG * HC);
+    auto load = [&](uint4 (&v)[NV]) {
       if constexpr (SRC == kSrcImage) {
-        gather_load(k + 2);   // stored after this tile's epilogue
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int q = lt + 128 * j, r = q / HC, c = q - r * HC;
+          const int y = at.ty * kConvTH - 1 + r, x = at.tx * kConvTW - 1 + c;
+          v[j] = make_uint4(0u, 0u, 0u, 0u);
+          if (q < HR * HC && y >= 0 && y < d.H && x >= 0 && x < d.W) {
+            const size_t src = ((size_t)at.b * io.H + 2 * y) * io.W + 2 * x;
+            v[j] = make_uint4(__float_as_uint(io.img[3 * src]), __float_as_uint(io.img[3 * src + 1]),
+                              __float_as_uint(io.img[3 * src + 2]), __float_as_uint(io.depth[src]));
+          }
+        }
       } else {
-        int b, y0, x0;
-        origin(k + 2, b, y0, x0);
-        load_halo_async<CG>(smem + (k & 1) * HALO, X, b, y0, x0, HR, HC, d.H, d.W);
-      }
-    }
-    // epilogue of tile k
-    float v[32];
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((k & 1) * 32);
-    if (COUT == 32) tc::tmem_ld32(taddr, v);
-    else tc::tmem_ld16(taddr, v);
-    if constexpr (DST == kDstCompose) {
-      if (inside) {
-        const int lv = io.levels[b * io.n_tiles + ((2 * y) / io.tile) * io.tiles_x + (2 * x) / io.tile];
-        if (lv < 4) {   // else every pixel of the block was rendered
-          // residual of colour c, sub-pixel s = 2 dy + dx: channel 4 c + s (12..15 unused)
-          float res[3][4];
+        const int x = at.tx * kConvTW - 1 + lc;
+        int y = at.ty * kConvTH - 1 + lrow;
+        const bool in_x = lrow < RSTEP && x >= 0 && x < d.W;
+        const uint4 *src = reinterpret_cast<const uint4 *>(X + (((ptrdiff_t)at.b * d.H + y) * d.W + x) * CIN + lg * 8);
 #pragma unroll
-          for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) res[c][q] = v[4 * c + q] + s_bias[4 * c + q];
-          compose_block(io.img, b, io.H, io.W, y, x, lv, res);
+        for (int j = 0; j < NV; ++j) {
+          v[j] = in_x && y >= 0 && y < d.H ? __ldg(src) : make_uint4(0u, 0u, 0u, 0u);
+          y += RSTEP;
+          src += (ptrdiff_t)RSTEP * d.W * CG;
         }
       }
-    } else if (inside) {
+      at.next();
+      at.next();
+    };
+    int sst = group, sph = 1;
+    auto store = [&](int k, const uint4 (&v)[NV]) {
+      if (k >= S && !tc::mbar_wait(&s_done[sst], sph) && lane == 0) atomicOr(status, kStatusTimeout);
+      uint8_t *hs = smem + sst * HALO;
+      if constexpr (SRC == kSrcImage) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int q = lt + 128 * j;
+          if (q < HR * HC)
+            *reinterpret_cast<uint4 *>(hs + q * 16) = block_operand(
+                make_float4(__uint_as_float(v[j].x), __uint_as_float(v[j].y), __uint_as_float(v[j].z),
+                            __uint_as_float(v[j].w)));
+        }
+      } else if (lrow < RSTEP) {
+#pragma unroll
+        for (int j = 0; j < NV; ++j)
+          *reinterpret_cast<uint4 *>(hs + lg * kConvPlane + ((lrow + j * RSTEP) * HC + lc) * 16) = v[j];
+      }
+      tc::fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&s_full[sst]);
+      sst += 2;
+      if (sst >= S) {
+        sst -= S;
+        sph ^= 1;
+      }
+    };
+    uint4 va[NV], vb[NV], vc[NV];
+    if (group < my_n) load(va);
+    if (group + 2 < my_n) load(vb);
+    for (int k = group; k < my_n; k += 6) {
+      if (k + 4 < my_n) load(vc);
+      store(k, va);
+      if (k + 2 >= my_n) break;
+      if (k + 6 < my_n) load(va);
+      store(k + 2, vb);
+      if (k + 4 >= my_n) break;
+      if (k + 8 < my_n) load(vb);
+      store(k + 4, vc);
+    }
+  } else {
+    const int group = warp >> 2, m = t & 127;   // accumulator row = output pixel of the tile
+    const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    uint4 rv[COUT / 8], mv[COUT / 8];
+    size_t pix = 0;
+    int b = 0, y = 0, x = 0;
+    bool inside = false;
+    TileWalk at(tiles_x, tiles_y);
+    if (group == 1) at.next();
+    auto prefetch = [&]() {   // the next tile of this group
+      b = at.b;
+      y = at.ty * kConvTH + m / kConvTW;
+      x = at.tx * kConvTW + (m % kConvTW);
+      inside = y < d.H && x < d.W;
+      pix = inside ? ((size_t)b * d.H + y) * d.W + x : 0;
 #pragma unroll
       for (int g = 0; g < COUT / 8; ++g) {
-        float o[8];
+        if (FLAGS & kEpiResid)
+          rv[g] = inside ? __ldg(reinterpret_cast<const uint4 *>(R + pix * COUT) + g) : make_uint4(0u, 0u, 0u, 0u);
+        if (FLAGS & kEpiMask)
+          mv[g] = inside ? __ldg(reinterpret_cast<const uint4 *>(Mk + pix * COUT) + g) : make_uint4(0u, 0u, 0u, 0u);
+      }
+      at.next();
+      at.next();
+    };
+    if (group < my_n) prefetch();
+    for (int k = group, st = group, ph = 0; k < my_n; k += 2) {
+      if (!tc::mbar_wait(&s_done[st], ph) && lane == 0) atomicOr(status, kStatusTimeout);
+      tc::fence_after_sync();
+      float v[32];
+      if (COUT == 32) tc::tmem_ld32(taddr + 32 * st, v);
+      else tc::tmem_ld16(taddr + 32 * st, v);
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&s_free[st]);
+      st += 2;
+      if (st >= S) {
+        st -= S;
+        ph ^= 1;
+      }
+      if constexpr ((FLAGS & kEpiBias) != 0) {
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          o[c] = v[g * 8 + c] + s_bias[g * 8 + c];
-          if (flags & kEpiRelu) o[c] = fmaxf(o[c], 0.0f);
-        }
-        if (flags & kEpiResid) {
-          const __nv_bfloat16 *rb = reinterpret_cast<const __nv_bfloat16 *>(&rv[g]);
-#pragma unroll
-          for (int c = 0; c < 8; ++c) o[c] += __bfloat162float(rb[c]);
-        }
-        if (flags & kEpiMask) {
-          const uint4 mv = __ldg(reinterpret_cast<const uint4 *>(Mk + pix * COUT) + g);
-          const __nv_bfloat16 *mb = reinterpret_cast<const __nv_bfloat16 *>(&mv);
-#pragma unroll
-          for (int c = 0; c < 8; ++c) o[c] = __bfloat162float(mb[c]) > 0.0f ? o[c] : 0.0f;
-        }
-        if (flags & kEpiF32) {
-          float4 *yo = reinterpret_cast<float4 *>(static_cast<float *>(Y) + pix * COUT + g * 8);
-          yo[0] = make_float4(o[0], o[1], o[2], o[3]);
-          yo[1] = make_float4(o[4], o[5], o[6], o[7]);
-        } else {
-          uint4 pk;
-          __nv_bfloat162 *p2 = reinterpret_cast<__nv_bfloat162 *>(&pk);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) p2[c] = __floats2bfloat162_rn(o[2 * c], o[2 * c + 1]);
-          reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(Y) + pix * COUT)[g] = pk;
+        for (int c = 0; c < COUT; c += 4) {
+          const float4 bv = *reinterpret_cast<const float4 *>(s_bias + c);
+          v[c] += bv.x;
+          v[c + 1] += bv.y;
+          v[c + 2] += bv.z;
+          v[c + 3] += bv.w;
         }
       }
+      if constexpr (DST == kDstCompose) {
+        if (inside) {
+          const int lv = io.levels[b * io.n_tiles + ((2 * y) / io.tile) * io.tiles_x + (2 * x) / io.tile];
+          if (lv < 4) {   // else every pixel of the block was rendered
+            // residual of colour c, sub-pixel s = 2 dy + dx: channel 4 c + s (12..15 unused)
+            float res[3][4];
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+              for (int q = 0; q < 4; ++q) res[c][q] = v[4 * c + q];
+            compose_block(io.img, b, io.H, io.W, y, x, lv, res);
+          }
+        }
+      } else {
+        uint4 out[4];   // the pixel's 64 bytes: 32 BF16 or 16 FP32 channels
+        static_assert(COUT * ((FLAGS & kEpiF32) ? 4 : 2) == 64 || DST == kDstCompose, "64 bytes a pixel");
+#pragma unroll
+        for (int g = 0; g < COUT / 8; ++g) {
+          float o[8];
+#pragma unroll
+          for (int c = 0; c < 8; ++c) o[c] = (FLAGS & kEpiRelu) ? fmaxf(v[g * 8 + c], 0.0f) : v[g * 8 + c];
+          if constexpr ((FLAGS & kEpiResid) != 0) {
+            const __nv_bfloat16 *rb = reinterpret_cast<const __nv_bfloat16 *>(&rv[g]);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) o[c] += __bfloat162float(rb[c]);
+          }
+          if constexpr ((FLAGS & kEpiMask) != 0) {
+            const __nv_bfloat16 *mb = reinterpret_cast<const __nv_bfloat16 *>(&mv[g]);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) o[c] = __bfloat162float(mb[c]) > 0.0f ? o[c] : 0.0f;
+          }
+          if constexpr ((FLAGS & kEpiF32) != 0) {
+            out[2 * g] = make_uint4(__float_as_uint(o[0]), __float_as_uint(o[1]), __float_as_uint(o[2]),
+                                    __float_as_uint(o[3]));
+            out[2 * g + 1] = make_uint4(__float_as_uint(o[4]), __float_as_uint(o[5]), __float_as_uint(o[6]),
+                                        __float_as_uint(o[7]));
+          } else {
+            __nv_bfloat162 *p2 = reinterpret_cast<__nv_bfloat162 *>(&out[g]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) p2[c] = __floats2bfloat162_rn(o[2 * c], o[2 * c + 1]);
+          }
+        }
+        // four lanes hold four pixels of one row: exchanged so that every store covers whole pixels
+        // (16 bytes a lane at a 64-byte stride would write every 32-byte sector in two halves)
+        transpose4(out);
+        const int xq = x & ~3;
+        const bool in_y = y < d.H;
+        uint4 *yo = static_cast<uint4 *>(Y) + (((size_t)b * d.H + y) * d.W + xq) * 4 + (lane & 3);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (in_y && xq + i < d.W) yo[4 * i] = out[i];
+      }
+      if (k + 2 < my_n) prefetch();
     }
-    if constexpr (SRC == kSrcImage) {
-      if (k + 2 < my_n) gather_store(smem + (k & 1) * HALO);
-    }
+    tc::fence_before_sync();
   }
-  tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, 64);
+  tc::fence_after_sync();
+  if (warp == 16) tc::tmem_dealloc(tmem, 512);
 }
 
 // The compact network's whole fill in one persistent kernel, per 16 x 16 block tile made of two
@@ -496,21 +589,12 @@ compact_fill_tc_kernel(ConvDims d, const uint4 *__restrict__ W0, const uint4 *__
       lv_next[h] = y < d.H && x < d.W ? lrow[(2 * x) >> lsh] : 4;
     }
   };
-  // the BF16 operand (r, g, b, depth / 8, then zeros: the conversion of block_input's first
-  // group) ...
+  // the BF16 operand ...
   auto store_operand = [&]() {
 #pragma unroll
     for (int j = 0; j < kGPer; ++j) {
       const int q = t + 128 * j;
-      if (q < HR * HC) {
-        uint4 lo;
-        __nv_bfloat162 *l2 = reinterpret_cast<__nv_bfloat162 *>(&lo);
-        l2[0] = __floats2bfloat162_rn(gv[j].x, gv[j].y);
-        l2[1] = __floats2bfloat162_rn(gv[j].z, gv[j].w * 0.125f);
-        l2[2] = __floats2bfloat162_rn(0.0f, 0.0f);
-        l2[3] = l2[2];
-        *reinterpret_cast<uint4 *>(halo + (size_t)q * 16) = lo;
-      }
+      if (q < HR * HC) *reinterpret_cast<uint4 *>(halo + (size_t)q * 16) = block_operand(gv[j]);
     }
   };
   // ... and the FP32 colours
@@ -691,7 +775,7 @@ compact_fill_tc_kernel(ConvDims d, const uint4 *__restrict__ W0, const uint4 *__
 // per tap row, (kx, cin) x cout, reads A three times (2.2 times the time per tile), and one CTA per
 // SM, because every CTA ends with the whole gradient in reductions (5 us of a launch at two per SM).
 // 32 -> 32 on 16 x 128 x 128 pixels under ncu: 318 us with both operands transposed into K-major
-// tiles by 2-byte stores and scalar reductions at a 36-byte stride; 20 us now.
+// tiles by 2-byte stores and scalar reductions at a 36-byte stride; 18 us now.
 constexpr int kWgTW = 8, kWgTH = 16;               // K = 128 pixels per tile
 constexpr int kWgStages = 4;
 constexpr int kWgThreads = 160;                    // four copying warps and the MMA warp
@@ -770,21 +854,22 @@ conv3x3_wgrad_tc_kernel(ConvDims d, const __nv_bfloat16 *__restrict__ X, const _
   const uint32_t tmem = s_tmem;
   pdl_begin();
   if (warp == 4) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = tc::idesc_bf16_f32(128, N) | tc::kIdescMnMajorA | tc::kIdescMnMajorB;
-      for (int k = 0; k < my_n; ++k) {
-        const int st = k % S;
-        if (!tc::mbar_wait(&s_full[st], (k / S) & 1)) atomicOr(status, kStatusTimeout);
-        tc::fence_after_sync();
-        const uint32_t b0 = tc::smem_u32(smem + st * STAGE), a0 = b0 + YOFF;
+    const bool leader = tc::elect_one();   // as in conv3x3_tc_kernel
+    constexpr uint32_t idesc = tc::idesc_bf16_f32(128, N) | tc::kIdescMnMajorA | tc::kIdescMnMajorB;
+    const uint32_t s0 = tc::smem_u32(smem);
+    for (int k = 0; k < my_n; ++k) {
+      const int st = k % S;
+      if (!tc::mbar_wait(&s_full[st], (k / S) & 1) && leader) atomicOr(status, kStatusTimeout);
+      tc::fence_after_sync();
+      const uint32_t b0 = s0 + st * STAGE, a0 = b0 + YOFF;
 #pragma unroll
-        for (int r = 0; r < kWgTH / 2; ++r)
-          tc::mma_bf16(tmem, tc::smem_desc(a0 + 2 * r * YROW, YROW, YC), tc::smem_desc(b0 + 2 * r * XROW, XROW, XP),
-                       idesc, k > 0 || r > 0);
-        tc::mma_commit(&s_empty[st]);
-      }
-      tc::mma_commit(&s_done);
+      for (int r = 0; r < kWgTH / 2; ++r)
+        tc::mma_bf16_if(leader, tmem, tc::smem_desc(a0 + 2 * r * YROW, YROW, YC),
+                        tc::smem_desc(b0 + 2 * r * XROW, XROW, XP), idesc, k > 0 || r > 0);
+      if (leader) tc::mma_commit(&s_empty[st]);
+      __syncwarp();
     }
+    if (leader) tc::mma_commit(&s_done);
     __syncwarp();
   } else {
     // threads 0..95 copy X (24 CG of them one row of the three copies), threads 96..127 dY (8 OG a
@@ -796,16 +881,16 @@ conv3x3_wgrad_tc_kernel(ConvDims d, const __nv_bfloat16 *__restrict__ X, const _
     const int lrow = mine_x ? lt / (CG * kWgTW * 3) : lt / (OG * kWgTW), lstep = mine_x ? 4 / CG : 4 / OG;
     const uint32_t ldst = mine_x ? (lkx * CG + lg) * XP + lrow * XROW + lc * 16
                                  : YOFF + lrow * YROW + lg * YC + lc * 16;
+    TileWalk at(tx_n, ty_n);
     for (int k = 0; k < my_n + 2; ++k) {
       const int st = k % S;
       if (k >= S && k < my_n && !tc::mbar_wait(&s_empty[st], (k / S - 1) & 1) && lane == 0)
         atomicOr(status, kStatusTimeout);
       if (k < my_n) {
-        const int tt = (int)blockIdx.x + k * (int)gridDim.x;
-        const int x0 = (tt % tx_n) * kWgTW, rest = tt / tx_n;
-        const int y0 = (rest % ty_n) * kWgTH, b = rest / ty_n;
+        const int x0 = at.tx * kWgTW, y0 = at.ty * kWgTH;
+        const ptrdiff_t img = (ptrdiff_t)at.b * d.H * d.W;
+        at.next();
         uint32_t dst = tc::smem_u32(smem + st * STAGE) + ldst;
-        const ptrdiff_t img = (ptrdiff_t)b * d.H * d.W;
         if (mine_x) {
           const int x = x0 - 1 + lkx + lc;
           const bool in_x = x >= 0 && x < d.W;
@@ -876,6 +961,7 @@ conv3x3_wgrad_tc_kernel(ConvDims d, const __nv_bfloat16 *__restrict__ X, const _
 // x0[b][y2][x2] = (r, g, b, depth / 8, 0 ...) of the top-left pixel of each 2x2 block.
 __global__ void gather_input_kernel(const float *__restrict__ img, const float *__restrict__ depth, int B,
                                     int H, int W, __nv_bfloat16 *__restrict__ x0) {
+  pdl_begin();
   const int H2 = (H + 1) / 2, W2 = (W + 1) / 2;
   const size_t n = (size_t)B * H2 * W2;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -911,6 +997,7 @@ __device__ __forceinline__ float base_px(const float *__restrict__ img, int b, i
 __global__ void loss_kernel(const float *__restrict__ r, const float *__restrict__ img,
                             const float *__restrict__ target, int B, int H, int W, float inv_count,
                             __nv_bfloat16 *__restrict__ g_r, float *__restrict__ loss_acc) {
+  pdl_begin();
   const int H2 = (H + 1) / 2, W2 = (W + 1) / 2;
   const size_t n = (size_t)B * H2 * W2;
   float acc = 0.0f;
@@ -953,6 +1040,7 @@ __global__ void loss_kernel(const float *__restrict__ r, const float *__restrict
 __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
                             float *__restrict__ v, int n, float lr, float b1, float b2, float eps,
                             float c1, float c2) {
+  pdl_begin();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.0f - b1) * gi;
@@ -969,6 +1057,7 @@ __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, 
 // other taps stay zero, so the 3x3 kernels train it unchanged.
 __global__ void pack_kernel(const float *__restrict__ w, int cin, int cout, int taps,
                             __nv_bfloat16 *__restrict__ fwd, __nv_bfloat16 *__restrict__ bwd) {
+  pdl_begin();
   const int n = cin * cout * taps;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int tap = taps == 9 ? i % 9 : 4, rest = taps == 9 ? i / 9 : i;
@@ -1029,6 +1118,7 @@ GradMap grad_map(int arch) {
 // The flat gradient, laid out as the parameters (W[cout][cin][taps] per layer, then the biases),
 // from the scratch gradient; a per-block layer takes the centre tap.
 __global__ void unpack_grads_kernel(GradMap m, const float *__restrict__ scratch, float *__restrict__ grads) {
+  pdl_begin();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m.n_params; i += gridDim.x * blockDim.x) {
     int l = m.n_layers - 1;
     if (i < m.b[0]) {
@@ -1105,25 +1195,23 @@ int ensure_acts(a3fr_cnn *n, size_t px) {
   return A3FR_OK;
 }
 
-template <int CIN, int COUT, int SRC = kSrcTensor, int DST = kDstTensor>
+template <int CIN, int COUT, int FLAGS, int SRC = kSrcTensor, int DST = kDstTensor>
 cudaError_t conv(const ConvDims &d, const __nv_bfloat16 *X, const __nv_bfloat16 *W, const float *bias,
-                 const __nv_bfloat16 *R, const __nv_bfloat16 *M, void *Y, int flags, uint32_t *status,
-                 cudaStream_t s, const FillIO &io = FillIO{}) {
+                 const __nv_bfloat16 *R, const __nv_bfloat16 *M, void *Y, uint32_t *status, cudaStream_t s,
+                 const FillIO &io = FillIO{}) {
   constexpr int smem = conv_smem_bytes<CIN, COUT>();
   static bool attr[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !attr[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv3x3_tc_kernel<CIN, COUT, SRC, DST>,
+    cudaError_t e = cudaFuncSetAttribute(conv3x3_tc_kernel<CIN, COUT, FLAGS, SRC, DST>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     attr[dev] = true;
   }
   const int tiles = d.B * ((d.W + kConvTW - 1) / kConvTW) * ((d.H + kConvTH - 1) / kConvTH);
-  const int grid = tiles < 152 * 5 ? tiles : 152 * 5;
-  conv3x3_tc_kernel<CIN, COUT, SRC, DST><<<grid, 128, smem, s>>>(d, X, reinterpret_cast<const uint4 *>(W), bias,
-                                                                 R, M, Y, flags, status, io);
-  return cudaGetLastError();
+  return launch_pdl(conv3x3_tc_kernel<CIN, COUT, FLAGS, SRC, DST>, tiles < 152 ? tiles : 152, kConvThreads, smem, s, d,
+                    X, reinterpret_cast<const uint4 *>(W), bias, R, M, Y, status, io);
 }
 
 cudaError_t compact_fill(const ConvDims &d, const a3fr_cnn *n, uint32_t *status, cudaStream_t s, const FillIO &io) {
@@ -1201,33 +1289,32 @@ int forward(a3fr_cnn *n, const float *img, const float *depth, int B, int H, int
   if (rc != A3FR_OK) return rc;
   const float *P = n->params;
   if (io) {
-    CNN_CHECK((conv<16, 32, kSrcImage>(d, nullptr, n->wf[0], P + bias_offset(A, 0), nullptr, nullptr, n->h[0],
-                                       kEpiBias | kEpiRelu, n->status, s, *io)));
+    CNN_CHECK((conv<16, 32, kBiasRelu, kSrcImage>(d, nullptr, n->wf[0], P + bias_offset(A, 0), nullptr, nullptr,
+                                                  n->h[0], n->status, s, *io)));
   } else {
-    gather_input_kernel<<<grid_1d(px), 256, 0, s>>>(img, depth, B, H, W, n->x0);
-    CNN_CHECK(cudaGetLastError());
-    CNN_CHECK((conv<16, 32>(d, n->x0, n->wf[0], P + bias_offset(A, 0), nullptr, nullptr, n->h[0],
-                            kEpiBias | kEpiRelu, n->status, s)));
+    CNN_CHECK(launch_pdl(gather_input_kernel, grid_1d(px), 256, 0, s, img, depth, B, H, W, n->x0));
+    CNN_CHECK((conv<16, 32, kBiasRelu>(d, n->x0, n->wf[0], P + bias_offset(A, 0), nullptr, nullptr, n->h[0], n->status,
+                                       s)));
   }
   if (A == A3FR_CNN_COMPACT) {
-    CNN_CHECK((conv<32, 32>(d, n->h[0], n->wf[1], P + bias_offset(A, 1), nullptr, nullptr, n->t[0],
-                            kEpiBias | kEpiRelu, n->status, s)));
-    CNN_CHECK((conv<32, 16>(d, n->t[0], n->wf[2], P + bias_offset(A, 2), nullptr, nullptr, n->r,
-                            kEpiBias | kEpiF32, n->status, s)));
+    CNN_CHECK((conv<32, 32, kBiasRelu>(d, n->h[0], n->wf[1], P + bias_offset(A, 1), nullptr, nullptr, n->t[0],
+                                       n->status, s)));
+    CNN_CHECK((conv<32, 16, kEpiBias | kEpiF32>(d, n->t[0], n->wf[2], P + bias_offset(A, 2), nullptr, nullptr, n->r,
+                                                n->status, s)));
     return A3FR_OK;
   }
   for (int b = 0; b < 4; ++b) {
-    CNN_CHECK((conv<32, 32>(d, n->h[b], n->wf[1 + 2 * b], P + bias_offset(A, 1 + 2 * b), nullptr, nullptr,
-                            n->t[b], kEpiBias | kEpiRelu, n->status, s)));
-    CNN_CHECK((conv<32, 32>(d, n->t[b], n->wf[2 + 2 * b], P + bias_offset(A, 2 + 2 * b), n->h[b], nullptr,
-                            n->h[b + 1], kEpiBias | kEpiResid, n->status, s)));
+    CNN_CHECK((conv<32, 32, kBiasRelu>(d, n->h[b], n->wf[1 + 2 * b], P + bias_offset(A, 1 + 2 * b), nullptr, nullptr,
+                                       n->t[b], n->status, s)));
+    CNN_CHECK((conv<32, 32, kEpiBias | kEpiResid>(d, n->t[b], n->wf[2 + 2 * b], P + bias_offset(A, 2 + 2 * b), n->h[b],
+                                                  nullptr, n->h[b + 1], n->status, s)));
   }
   if (io) {
-    CNN_CHECK((conv<32, 16, kSrcTensor, kDstCompose>(d, n->h[4], n->wf[9], P + bias_offset(A, 9), nullptr, nullptr,
-                                                     nullptr, kEpiBias, n->status, s, *io)));
+    CNN_CHECK((conv<32, 16, kEpiBias, kSrcTensor, kDstCompose>(d, n->h[4], n->wf[9], P + bias_offset(A, 9), nullptr,
+                                                               nullptr, nullptr, n->status, s, *io)));
   } else {
-    CNN_CHECK((conv<32, 16>(d, n->h[4], n->wf[9], P + bias_offset(A, 9), nullptr, nullptr, n->r,
-                            kEpiBias | kEpiF32, n->status, s)));
+    CNN_CHECK((conv<32, 16, kEpiBias | kEpiF32>(d, n->h[4], n->wf[9], P + bias_offset(A, 9), nullptr, nullptr, n->r,
+                                                n->status, s)));
   }
   return A3FR_OK;
 }
@@ -1239,35 +1326,35 @@ int backward(a3fr_cnn *n, const float *img, const float *target, int B, int H, i
   const int A = n->arch;
   CNN_CHECK(cudaMemsetAsync(n->wscratch, 0, sizeof(float) * scratch_offset(A, n_layers(A)), s));
   CNN_CHECK(cudaMemsetAsync(n->loss_acc, 0, sizeof(float), s));
-  loss_kernel<<<grid_1d(px), 256, 0, s>>>(n->r, img, target, B, H, W, 1.0f / (3.0f * B * H * W), n->g_r,
-                                          n->loss_acc);
-  CNN_CHECK(cudaGetLastError());
+  CNN_CHECK(launch_pdl(loss_kernel, grid_1d(px), 256, 0, s, n->r, img, target, B, H, W, 1.0f / (3.0f * B * H * W),
+                       n->g_r, n->loss_acc));
   if (A == A3FR_CNN_COMPACT) {
     // r = W2 t + b2;  t = ReLU(W1 h + b1);  h = ReLU(conv0(x0) + b0)
     CNN_CHECK((wgrad<32, 16>(n, 2, d, n->t[0], n->g_r, s)));
-    CNN_CHECK((conv<16, 32>(d, n->g_r, n->wb[2], nullptr, nullptr, n->t[0], n->gA, kEpiMask, n->status, s)));
+    CNN_CHECK((conv<16, 32, kEpiMask>(d, n->g_r, n->wb[2], nullptr, nullptr, n->t[0], n->gA, n->status, s)));
     CNN_CHECK((wgrad<32, 32>(n, 1, d, n->h[0], n->gA, s)));
-    CNN_CHECK((conv<32, 32>(d, n->gA, n->wb[1], nullptr, nullptr, n->h[0], n->gB, kEpiMask, n->status, s)));
+    CNN_CHECK((conv<32, 32, kEpiMask>(d, n->gA, n->wb[1], nullptr, nullptr, n->h[0], n->gB, n->status, s)));
     CNN_CHECK((wgrad<16, 32>(n, 0, d, n->x0, n->gB, s)));
   } else {
     CNN_CHECK((wgrad<32, 16>(n, 9, d, n->h[4], n->g_r, s)));
-    CNN_CHECK((conv<16, 32>(d, n->g_r, n->wb[9], nullptr, nullptr, nullptr, n->gA, 0, n->status, s)));
+    CNN_CHECK((conv<16, 32, 0>(d, n->g_r, n->wb[9], nullptr, nullptr, nullptr, n->gA, n->status, s)));
     __nv_bfloat16 *cur = n->gA, *nxt = n->gB;
     for (int b = 3; b >= 0; --b) {
       const int l2 = 2 + 2 * b, l1 = 1 + 2 * b;
       CNN_CHECK((wgrad<32, 32>(n, l2, d, n->t[b], cur, s)));
-      CNN_CHECK((conv<32, 32>(d, cur, n->wb[l2], nullptr, nullptr, n->t[b], n->gT, kEpiMask, n->status, s)));
+      CNN_CHECK((conv<32, 32, kEpiMask>(d, cur, n->wb[l2], nullptr, nullptr, n->t[b], n->gT, n->status, s)));
       CNN_CHECK((wgrad<32, 32>(n, l1, d, n->h[b], n->gT, s)));
-      CNN_CHECK((conv<32, 32>(d, n->gT, n->wb[l1], nullptr, cur, b == 0 ? n->h[0] : nullptr, nxt,
-                              kEpiResid | (b == 0 ? kEpiMask : 0), n->status, s)));
+      if (b == 0)
+        CNN_CHECK((conv<32, 32, kEpiResid | kEpiMask>(d, n->gT, n->wb[l1], nullptr, cur, n->h[0], nxt, n->status, s)));
+      else
+        CNN_CHECK((conv<32, 32, kEpiResid>(d, n->gT, n->wb[l1], nullptr, cur, nullptr, nxt, n->status, s)));
       __nv_bfloat16 *tmp = cur;
       cur = nxt;
       nxt = tmp;
     }
     CNN_CHECK((wgrad<16, 32>(n, 0, d, n->x0, cur, s)));
   }
-  unpack_grads_kernel<<<grid_1d(n_params(A)), 256, 0, s>>>(grad_map(A), n->wscratch, n->grads);
-  CNN_CHECK(cudaGetLastError());
+  CNN_CHECK(launch_pdl(unpack_grads_kernel, grid_1d(n_params(A)), 256, 0, s, grad_map(A), n->wscratch, n->grads));
   return A3FR_OK;
 }
 
