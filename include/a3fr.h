@@ -251,8 +251,9 @@ int a3fr_set_batch(a3fr_scene *scene, int batch_mult);
  * the depth-ordered entries cut into chunks, per-chunk tile counts and start slots, every
  * instance placed at its slot by ordered ranks (no sort over the instances).  SORTED: tile
  * counts, emit of the depth-ordered instances, a stable radix sort by tile.  AUTO (default):
- * DIRECT up to 6,144 tiles over all eyes, SORTED above (where it is faster).  Changing it invalidates the scene's buffers (the next render reallocates);
- * synchronous.  Invalid mode: A3FR_ERR_INVALID_ARG. */
+ * DIRECT up to 6,144 tiles over all eyes, and up to 16,384 while tiles x entries (Gaussians times
+ * eyes) is at most 1.6e10; SORTED above (where it is faster).  Changing it invalidates the scene's
+ * buffers (the next render reallocates); synchronous.  Invalid mode: A3FR_ERR_INVALID_ARG. */
 #define A3FR_BINNING_AUTO 0
 #define A3FR_BINNING_DIRECT 1
 #define A3FR_BINNING_SORTED 2

@@ -64,8 +64,7 @@ struct a3fr_scene {
   uint32_t *dvals[2] = {nullptr, nullptr};   // depth-sorted entries e * n + i
   uint2 *ranges = nullptr;
   uint32_t *bin_h = nullptr;                 // per-chunk tile counts, then starts (binning.cu)
-  // the sort-based binning (binning_sorted.cu), for renders with more than
-  // kBinDirectMaxTiles tiles: difference grids, instance tile keys, the sort's second buffers
+  // the sort-based binning (binning_sorted.cu; see auto_bin_direct): difference grids, instance tile keys, the sort's second buffers
   int binning = A3FR_BINNING_AUTO;
   bool sorted_bin = false;
   uint32_t *tile_partials = nullptr;
@@ -159,11 +158,18 @@ int n_eyes_of(const a3fr_scene *s) { return s->cam_set[1] ? 2 : (s->cam_set[0] ?
 
 constexpr int kDepthPasses = 4;   // 32-bit depth keys, 8-bit digits
 
-// AUTO binning: direct placement up to this many tiles (all eyes), the sort-based binning
-// above.  Each direct-binning warp walks one chunk of entries serially; with many tiles the
-// chunk table (chunks x tiles) caps the chunk count, the chains grow and the stable radix
-// sort by tile is faster (3M clustered stereo 2064x2208, 8,970 tiles: 0.54 vs 0.80 ms).
-constexpr int kBinDirectMaxTiles = 6144;
+// AUTO binning: direct placement up to kBinDirectMaxTiles tiles (all eyes), and beyond that for up to
+// kBinDirectMaxTilesBig tiles while tiles x entries stays below kBinDirectMaxWork; else the sort-based
+// binning.  Each direct-binning warp walks one chunk of entries serially, and the chunk table
+// (chunks x tiles) caps the chunk count: with many tiles and entries the chains grow and the stable
+// radix sort by tile is faster.  Tile counts to placed instances, direct / sorted (us; uniform scenes):
+// 8,160 tiles 500k entries 147 / 193, 1M 260 / 319, 2M 618 / 578; 16,320 tiles 100k 70 / 97,
+// 1M 303 / 336, 2M 706 / 601; 17,802 tiles 500k 244 / 224; 8,970 tiles 6M (clustered) 726 / 535.
+constexpr long long kBinDirectMaxTiles = 6144, kBinDirectMaxTilesBig = 16384, kBinDirectMaxWork = 16000000000ll;
+
+bool auto_bin_direct(long long tiles, long long entries) {
+  return tiles <= kBinDirectMaxTiles || (tiles <= kBinDirectMaxTilesBig && tiles * entries <= kBinDirectMaxWork);
+}
 
 int tile_bits_for(int n_ranges) {
   int bits = 1;
@@ -290,7 +296,7 @@ int ensure_frame_buffers(a3fr_scene *s, int eyes, int W, int H) {
     A3FR_CHECK(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const int tx = (W + tile - 1) / tile, ty = (H + tile - 1) / tile;
     s->sorted_bin = s->binning == A3FR_BINNING_SORTED ||
-                    (s->binning == A3FR_BINNING_AUTO && (long long)eyes * tx * ty > kBinDirectMaxTiles);
+                    (s->binning == A3FR_BINNING_AUTO && !auto_bin_direct((long long)eyes * tx * ty, (long long)eyes * n));
     const size_t need = s->sorted_bin ? tile_scan_smem_bytes(eyes, tx, ty) + 9216 : bin_smem_bytes(eyes, tx, ty);
     if (need > (size_t)max_optin) return A3FR_ERR_INVALID_ARG;
   }
@@ -503,7 +509,7 @@ int size_instances(a3fr_scene *s, cudaStream_t stream) {
   return A3FR_OK;
 }
 
-// The sort-based binning (renders with more than kBinDirectMaxTiles tiles): tile counts ->
+// The sort-based binning (see auto_bin_direct): tile counts ->
 // ranges and the tile sort's histograms, emit of the depth-ordered instances, stable
 // onesweep by tile index.  The sort's result lands in s->vals.
 int enqueue_bin_sorted(a3fr_scene *s, int eyes, Entries entries, const FrameLayout &L,

@@ -1,0 +1,50 @@
+"""Direct placement against the sort-based binning: the same keys, values and tile ranges, bit for bit,
+where the direct one's bands and steps have their edges -- one row of tiles, fewer rows than bands, odd
+rows over two eyes, the most tiles AUTO gives it (four bands), Gaussians that cover every tile, tiles
+that several Gaussians of one step share, and a capacity that cuts the lists off."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import paper_2507_04147_gb300 as a3fr
+from paper_2507_04147_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("w,h,eyes,tile,n,log_scale,capacity", [
+    (333, 16, 1, 16, 3_000, -3.0, 0),       # one row of tiles: one band
+    (16, 700, 2, 32, 2_000, -2.0, 0),       # one column, 2 x 22 rows
+    (40, 40, 1, 16, 5_000, -1.0, 0),        # nine tiles: every step shares tiles
+    (517, 389, 2, 16, 4_001, -3.5, 0),      # odd rows per eye
+    (2048, 2048, 1, 16, 20_000, -4.0, 0),   # 16,384 tiles, four bands
+    (640, 480, 2, 16, 300, 1.5, 0),         # Gaussians over the whole image
+    (517, 389, 1, 16, 4_001, -3.5, 5_000),  # capacity reached
+])
+def test_direct_equals_sorted(w, h, eyes, tile, n, log_scale, capacity):
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    sc = synth.uniform_scene(n, 0, seed=n, log_scale_mean=log_scale)
+    sc = dataclasses.replace(sc, means=np.where(np.arange(n)[:, None] % 9 == 4, -sc.means, sc.means))   # some behind
+    cams = synth.stereo_cameras(w, h) if eyes == 2 else [synth.pinhole_camera(w, h)]
+    got = []
+    for mode in (a3fr.BINNING_DIRECT, a3fr.BINNING_SORTED):
+        s = a3fr.Scene.from_numpy(sc, instance_capacity=capacity, tile=tile)
+        s.set_binning(mode)
+        for e, c in enumerate(cams):
+            s.set_camera(e, c)
+        img = s.render_full().cpu().numpy()
+        st = s.stats()
+        got.append((s.buffer(a3fr.BUF_KEYS, torch.int64).cpu().numpy(), s.buffer(a3fr.BUF_VALUES, torch.int32).cpu().numpy(),
+                    s.buffer(a3fr.BUF_RANGES, torch.int32).cpu().numpy(), img if not capacity else np.zeros(1)))
+        assert st["status"] == (a3fr.STATUS_CAPACITY if capacity else 0)
+        assert st["instances"] > 0
+        s.close()
+    if capacity:   # both keep the first `capacity` slots' worth of whole lists; compare what lies below it
+        ends = got[0][2].reshape(-1, 2)
+        assert np.array_equal(ends, got[1][2].reshape(-1, 2))
+        return
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
