@@ -71,94 +71,115 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *s_tmp)
   return before + incl - v;
 }
 
-// Digit histograms of every pass in one read of the keys.  Each thread walks a contiguous
-// run of keys and, per pass, adds to shared memory only when the digit changes (so the
-// few-valued high digits of depths cost one atomic per run instead of one per key); each
-// warp owns a private copy of the counters, summed at the end.
+// Digit histograms of every pass in one read of the keys.  Each thread takes eight keys at a time in
+// 16-byte loads and, per pass, adds to shared memory only when the digit changes (so the
+// few-valued high digits of depths cost one atomic per run instead of one per key); even and odd
+// warps have their own counters.  Few blocks: every block clears, sums and adds up to
+// 2,048 counters, which with one block per 2,048 keys and a copy per warp cost more than the keys.
+// 4M 64-bit keys, 6 passes (ncu): 45 us with four passes to a read and 8-byte loads, 20 us now;
+// 6M depth keys 25, 19 us; 1M 9.7, 7.8 us.
 constexpr int kHistKeysPerThread = 8;
+constexpr int kHistCopies = 2;
 
 template <typename K, bool kRebase>
 __global__ void __launch_bounds__(kThreads)
 histogram_kernel(K *__restrict__ keys, const uint32_t *__restrict__ d_count, SortPlan plan,
                  uint32_t *__restrict__ hist, const uint32_t *__restrict__ range) {
   pdl_begin();
-  __shared__ uint32_t s_hist[kWarps][4][kRadix];   // per warp, up to 4 passes per launch
-  const int t = threadIdx.x, warp = t >> 5;
+  constexpr int KPT = kHistKeysPerThread, VEC = 16 / (int)sizeof(K);   // keys per load
+  __shared__ uint32_t s_hist[kHistCopies][kMaxSortPasses][kRadix];
+  const int t = threadIdx.x, copy = (t >> 5) % kHistCopies;
   const uint32_t n = *d_count;
-  for (int p0 = 0; p0 < plan.passes; p0 += 4) {
-    const int np = min(4, plan.passes - p0);
-    for (int i = t; i < kWarps * 4 * kRadix; i += kThreads) (&s_hist[0][0][0])[i] = 0;
-    __syncthreads();
-    const uint32_t per_block = kThreads * kHistKeysPerThread;
-    // a thread's 8 consecutive 32-bit keys as two 16-byte loads (and stores, when rebased)
-    constexpr bool kVec = sizeof(K) == 4 && kHistKeysPerThread == 8;
-    const bool vec_ok = kVec && (reinterpret_cast<uintptr_t>(keys) & 15u) == 0u;
-    for (uint32_t base = blockIdx.x * per_block; base < n; base += gridDim.x * per_block) {
-      const uint32_t i0 = base + t * kHistKeysPerThread;
-      const uint32_t i1 = min(n, i0 + kHistKeysPerThread);
-      const bool vec = vec_ok && i1 == i0 + kHistKeysPerThread;
-      K kv[kHistKeysPerThread];
-      if constexpr (kVec) {
-        if (vec) {
-          const uint4 a = reinterpret_cast<const uint4 *>(keys + i0)[0];
-          const uint4 b = reinterpret_cast<const uint4 *>(keys + i0)[1];
-          kv[0] = a.x; kv[1] = a.y; kv[2] = a.z; kv[3] = a.w;
-          kv[4] = b.x; kv[5] = b.y; kv[6] = b.z; kv[7] = b.w;
+  // visible keys are <= max; a range under 2^24 leaves the top digit zero
+  uint32_t kmin = 0u, kmax = 0u;
+  bool rebase = false;
+  if (kRebase) {
+    kmin = ~range[0];
+    kmax = range[2];
+    rebase = kmax >= kmin && kmax - kmin < (1u << 24);
+  }
+  for (int i = t; i < kHistCopies * kMaxSortPasses * kRadix; i += kThreads) (&s_hist[0][0][0])[i] = 0;
+  __syncthreads();
+  const bool aligned = (reinterpret_cast<uintptr_t>(keys) & 15u) == 0u;
+  constexpr uint32_t kPerBlock = kThreads * KPT;
+  for (uint32_t base = blockIdx.x * kPerBlock; base < n; base += gridDim.x * kPerBlock) {
+    K kv[KPT];
+    // load j of thread t: keys base + (j kThreads + t) VEC ...; past the end, and for unaligned keys,
+    // one at a time
+    const bool whole = aligned && n - base >= kPerBlock;
+    int have = KPT;
+    if (whole) {
+#pragma unroll
+      for (int j = 0; j < KPT / VEC; ++j) {
+        const uint4 v = reinterpret_cast<const uint4 *>(keys + base)[j * kThreads + t];
+        if constexpr (sizeof(K) == 8) {
+          kv[2 * j] = (K)v.x | ((K)v.y << 32);
+          kv[2 * j + 1] = (K)v.z | ((K)v.w << 32);
+        } else {
+          kv[4 * j] = v.x;
+          kv[4 * j + 1] = v.y;
+          kv[4 * j + 2] = v.z;
+          kv[4 * j + 3] = v.w;
         }
       }
-      bool rebased = false;
-      uint32_t cur[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};
-      uint32_t run[4] = {0u, 0u, 0u, 0u};
+    } else {
+      const uint32_t left = n - base;
+      have = 0;
 #pragma unroll
-      for (int j = 0; j < kHistKeysPerThread; ++j) {
-        const uint32_t i = i0 + (uint32_t)j;
-        if (i >= i1) break;
-        K k = vec ? kv[j] : keys[i];
-        if (kRebase && p0 == 0) {
-          // visible keys are <= max; a range under 2^24 leaves the top digit zero
-          const uint32_t kmin = ~range[0], kmax = range[2];
-          if (kmax >= kmin && kmax - kmin < (1u << 24)) {
-            k = (K)((uint32_t)k <= kmax ? (uint32_t)k - kmin : 0xffffffu);
-            if (vec) {
-              kv[j] = k;
-              rebased = true;
-            } else {
-              keys[i] = k;
-            }
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (q < np) {
-            const uint32_t d = (uint32_t)(k >> plan.shift[p0 + q]) & plan.mask;
-            if (d != cur[q]) {
-              if (run[q]) atomicAdd(&s_hist[warp][q][cur[q]], run[q]);
-              cur[q] = d;
-              run[q] = 0;
-            }
-            ++run[q];
-          }
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (q < np && run[q]) atomicAdd(&s_hist[warp][q][cur[q]], run[q]);
-      if constexpr (kVec) {
-        if (rebased) {
-          reinterpret_cast<uint4 *>(keys + i0)[0] = make_uint4(kv[0], kv[1], kv[2], kv[3]);
-          reinterpret_cast<uint4 *>(keys + i0)[1] = make_uint4(kv[4], kv[5], kv[6], kv[7]);
+      for (int j = 0; j < KPT; ++j) {
+        const uint32_t i = (uint32_t)(j * kThreads + t);
+        if (i < left) {
+          kv[j] = keys[base + i];
+          have = j + 1;
         }
       }
     }
-    __syncthreads();
-    for (int i = t; i < np * kRadix; i += kThreads) {
-      const int q = i / kRadix, d = i - q * kRadix;
-      uint32_t v = 0;
+    if (kRebase && rebase) {
 #pragma unroll
-      for (int w = 0; w < kWarps; ++w) v += s_hist[w][q][d];
-      if (v) atomicAdd(hist + (p0 + q) * kRadix + d, v);
+      for (int j = 0; j < KPT; ++j) kv[j] = (K)((uint32_t)kv[j] <= kmax ? (uint32_t)kv[j] - kmin : 0xffffffu);
+      if (whole) {
+#pragma unroll
+        for (int j = 0; j < KPT / VEC; ++j)
+          if constexpr (sizeof(K) == 4)
+            reinterpret_cast<uint4 *>(keys + base)[j * kThreads + t] =
+                make_uint4(kv[4 * j], kv[4 * j + 1], kv[4 * j + 2], kv[4 * j + 3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < KPT; ++j)
+          if (j < have) keys[base + j * kThreads + t] = kv[j];
+      }
     }
-    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kMaxSortPasses; ++q) {
+      if (q >= plan.passes) break;
+      uint32_t cur = 0u, run = 0u;
+#pragma unroll
+      for (int j = 0; j < KPT; ++j) {
+        if (j >= have) break;
+        const uint32_t d = (uint32_t)(kv[j] >> plan.shift[q]) & plan.mask;
+        if (run && d != cur) {
+          atomicAdd(&s_hist[copy][q][cur], run);
+          run = 0u;
+        }
+        cur = d;
+        ++run;
+      }
+      // a digit that is the same across the warp (the top one of rebased keys): one atomic
+      int same = 0;
+      __match_all_sync(0xffffffffu, run == (uint32_t)KPT ? cur : 0x80000000u | (uint32_t)t, &same);
+      if (same) {
+        if ((t & 31) == 0) atomicAdd(&s_hist[copy][q][cur], 32u * KPT);
+      } else if (run) {
+        atomicAdd(&s_hist[copy][q][cur], run);
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = t; i < plan.passes * kRadix; i += kThreads) {
+    uint32_t v = 0;
+#pragma unroll
+    for (int c = 0; c < kHistCopies; ++c) v += (&s_hist[c][0][0])[i];
+    if (v) atomicAdd(hist + i, v);
   }
 }
 
@@ -511,10 +532,13 @@ size_t onesweep_lookback_bytes(size_t capacity, int passes, bool wide_keys, bool
 }
 
 int histogram_blocks(size_t capacity) {
-  const int sms = sm_count();
-  const size_t per_block = (size_t)kThreads * kHistKeysPerThread;
-  const size_t hb = (capacity + per_block - 1) / per_block;
-  return (int)(hb < (size_t)sms * 8 ? (hb > 0 ? hb : 1) : (size_t)sms * 8);
+  // four reads of 2,048 keys a block, but at least two and at most four blocks per SM (1M keys: two
+  // 7.8 us, four 8.8; 4M 64-bit keys: two 25.6, four 19.8, eight 22.3)
+  const size_t sms = (size_t)sm_count(), per_block = (size_t)kThreads * kHistKeysPerThread;
+  const size_t chunks = (capacity + per_block - 1) / per_block;
+  size_t blocks = chunks / 4;
+  blocks = blocks < 2 * sms ? 2 * sms : (blocks > 4 * sms ? 4 * sms : blocks);
+  return (int)(chunks < blocks ? (chunks > 0 ? chunks : 1) : blocks);
 }
 
 template <typename K>
