@@ -241,11 +241,12 @@ struct LanePixels {
 };
 
 // One item, by the whole CTA: the Gaussians of a tile's list blended into every lane's pixels.
-// Without the auxiliary outputs a finished pixel is marked by T = 0 (a live pixel keeps
-// T >= 1e-4): skipped Gaussians then blend with alpha 0, which leaves T and the colour bit for
-// bit as they were, and every later Gaussian of a finished pixel stops with weight 0.  With them
-// the loop also keeps the final transmittance, the last contributor and the evaluation and blend
-// counts.  inherit: pixel 0 is the top-left one of the block at (px0, py0), and the labels from
+// A finished pixel is marked by T = 0 (a live pixel keeps T >= 1e-4): skipped Gaussians then blend
+// with alpha 0, which leaves T and the colour bit for bit as they were, and every later Gaussian of
+// a finished pixel stops with weight 0.  With the auxiliary outputs a finished pixel keeps its final
+// transmittance negated instead, and the loop also keeps the last contributor and the evaluation and
+// blend counts: one select each and no flags (500k stereo 158 -> 137 us under ncu; 16-pixel tiles, at
+// 5 CTAs per SM, 1M at 1024 x 1024 76 -> 71 us).  inherit: pixel 0 is the top-left one of the block at (px0, py0), and the labels from
 // hi on take its value.
 template <int P, bool kAux, int kMult>
 __device__ __forceinline__ void render_pixels(ItemSmem<kMult> &sm, const CompositeParams &p, const float *rec,
@@ -264,20 +265,27 @@ __device__ __forceinline__ void render_pixels(ItemSmem<kMult> &sm, const Composi
   const float *rec_eye = rec + (size_t)eye * n * kRec;
 
   float T[P], C0[P], C1[P], C2[P], Z[P];
-  uint32_t last[P], stop[P];
-  bool done[P];
+  uint32_t last[P], stop[P], blended = 0;
 #pragma unroll
   for (int k = 0; k < P; ++k) {
-    T[k] = kAux || inside[k] ? 1.0f : 0.0f;
+    T[k] = inside[k] ? 1.0f : (kAux ? -1.0f : 0.0f);
     C0[k] = C1[k] = C2[k] = Z[k] = 0.0f;
     last[k] = stop[k] = 0u;
-    done[k] = !inside[k];
   }
   auto all_done = [&]() {
     bool a = true;
 #pragma unroll
-    for (int k = 0; k < P; ++k) a = a && (kAux ? done[k] : T[k] == 0.0f);
+    for (int k = 0; k < P; ++k) a = a && T[k] <= 0.0f;
     return a;
+  };
+  // the auxiliary outputs' bookkeeping of pixel k at list position pos, and its new T: alpha a is
+  // blended unless it would end the pixel or the pixel had ended (tt, T (1 - a), below 1e-4 or negative)
+  auto note = [&](int k, float a, float tt, uint32_t pos) {
+    const bool go = tt >= 0.0001f, upd = go && a > 0.0f;
+    last[k] = upd ? pos : last[k];
+    blended += upd ? 1u : 0u;
+    stop[k] = !go && T[k] > 0.0f ? pos : stop[k];
+    T[k] = go ? tt : -fabsf(T[k]);
   };
   for (uint32_t start = range.x; start < range.y; start += NB) {
     const bool wdone = __all_sync(0xffffffffu, all_done());
@@ -355,7 +363,7 @@ __device__ __forceinline__ void render_pixels(ItemSmem<kMult> &sm, const Composi
           const float2 cz = sm.cz[e];
           const float4 rgb = sm.rgb[e];
           const uint32_t pos = pos0 + (uint32_t)e;
-          if constexpr (!kAux && P >= 2) {
+          if constexpr (P >= 2) {
             // pixel pairs (0, 1) and (2, 3): the same operations as the scalar loop below, two
             // pixels per instruction wherever both take the same one
             const f32x2 gx = f2_pack(geo.x, geo.x), gy = f2_pack(geo.y, geo.y);
@@ -387,50 +395,13 @@ __device__ __forceinline__ void render_pixels(ItemSmem<kMult> &sm, const Composi
               f2_unpack(f2_fma(cr, w2, f2_pack(C0[k], C0[k + 1])), C0[k], C0[k + 1]);
               f2_unpack(f2_fma(cg, w2, f2_pack(C1[k], C1[k + 1])), C1[k], C1[k + 1]);
               f2_unpack(f2_fma(cbl, w2, f2_pack(C2[k], C2[k + 1])), C2[k], C2[k + 1]);
-              f2_unpack(f2_mul(tt2, keep), T[k], T[k + 1]);
-            }
-          }
-          if constexpr (kAux && P >= 2) {
-            // the same pairs with the auxiliary outputs: the arithmetic packed, the bookkeeping
-            // (done, last contributor, stop position, blend count) per pixel
-            const f32x2 gx = f2_pack(geo.x, geo.x), gy = f2_pack(geo.y, geo.y);
-            const f32x2 ca = f2_pack(geo.z, geo.z), cb = f2_pack(geo.w, geo.w), cc = f2_pack(cz.x, cz.x);
-            const f32x2 op = f2_pack(rgb.w, rgb.w);
-            const f32x2 cr = f2_pack(rgb.x, rgb.x), cg = f2_pack(rgb.y, rgb.y), cbl = f2_pack(rgb.z, rgb.z);
-            const f32x2 cdz = f2_pack(cz.y, cz.y);
-            const f32x2 one = f2_pack(1.0f, 1.0f), mone = f2_pack(-1.0f, -1.0f);
-#pragma unroll
-            for (int k = 0; k + 1 < P; k += 2) {
-              const f32x2 dx = f2_add(gx, f2_pack(-fpx[k], -fpx[k + 1]));
-              const f32x2 dy = f2_add(gy, f2_pack(-fpy[k], -fpy[k + 1]));
-              const f32x2 pw2 = f2_fma(f2_fma(ca, dx, f2_mul(cb, dy)), dx, f2_mul(f2_mul(cc, dy), dy));
-              float pw0, pw1;
-              f2_unpack(pw2, pw0, pw1);
-              float oe0, oe1;
-              f2_unpack(f2_mul(op, f2_pack(ex2_approx(pw0), ex2_approx(pw1))), oe0, oe1);
-              const float al0 = fminf(0.99f, oe0), al1 = fminf(0.99f, oe1);
-              const f32x2 al2 = f2_pack(al0, al1), t2 = f2_pack(T[k], T[k + 1]);
-              float tt0, tt1, at0, at1;
-              f2_unpack(f2_mul(t2, f2_fma(al2, mone, one)), tt0, tt1);   // T (1 - alpha)
-              f2_unpack(f2_mul(al2, t2), at0, at1);
-              const bool ok0 = !done[k] && pw0 <= 0.0f && al0 >= 1.0f / 255.0f;
-              const bool ok1 = !done[k + 1] && pw1 <= 0.0f && al1 >= 1.0f / 255.0f;
-              const bool fin0 = ok0 && tt0 < 0.0001f, fin1 = ok1 && tt1 < 0.0001f;
-              const bool upd0 = ok0 && !fin0, upd1 = ok1 && !fin1;
-              const f32x2 w2 = f2_pack(upd0 ? at0 : 0.0f, upd1 ? at1 : 0.0f);
-              f2_unpack(f2_fma(cr, w2, f2_pack(C0[k], C0[k + 1])), C0[k], C0[k + 1]);
-              f2_unpack(f2_fma(cg, w2, f2_pack(C1[k], C1[k + 1])), C1[k], C1[k + 1]);
-              f2_unpack(f2_fma(cbl, w2, f2_pack(C2[k], C2[k + 1])), C2[k], C2[k + 1]);
-              f2_unpack(f2_fma(cdz, w2, f2_pack(Z[k], Z[k + 1])), Z[k], Z[k + 1]);
-              bl += (upd0 ? 1u : 0u) + (upd1 ? 1u : 0u);
-              T[k] = upd0 ? tt0 : T[k];
-              T[k + 1] = upd1 ? tt1 : T[k + 1];
-              last[k] = upd0 ? pos : last[k];
-              last[k + 1] = upd1 ? pos : last[k + 1];
-              stop[k] = fin0 ? pos : stop[k];
-              stop[k + 1] = fin1 ? pos : stop[k + 1];
-              done[k] = done[k] || fin0;
-              done[k + 1] = done[k + 1] || fin1;
+              if constexpr (kAux) {
+                f2_unpack(f2_fma(f2_pack(cz.y, cz.y), w2, f2_pack(Z[k], Z[k + 1])), Z[k], Z[k + 1]);
+                note(k, a0, tt0, pos);
+                note(k + 1, a1, tt1, pos);
+              } else {
+                f2_unpack(f2_mul(tt2, keep), T[k], T[k + 1]);
+              }
             }
           }
 #pragma unroll
@@ -441,29 +412,17 @@ __device__ __forceinline__ void render_pixels(ItemSmem<kMult> &sm, const Composi
             const float dx = __fsub_rn(geo.x, fpx[k]), dy = __fsub_rn(geo.y, fpy[k]);
             const float pw = falloff_log2(geo.z, geo.w, cz.x, dx, dy);
             const float alpha = blend_alpha(rgb.w, pw);
+            const float a = (pw <= 0.0f && alpha >= 1.0f / 255.0f) ? alpha : 0.0f;
+            const float tt = __fmul_rn(T[k], __fsub_rn(1.0f, a));
+            const bool fin = tt < 0.0001f;   // this Gaussian would end the pixel, or it ended
+            const float w = fin ? 0.0f : __fmul_rn(a, T[k]);
+            C0[k] = __fmaf_rn(rgb.x, w, C0[k]);
+            C1[k] = __fmaf_rn(rgb.y, w, C1[k]);
+            C2[k] = __fmaf_rn(rgb.z, w, C2[k]);
             if constexpr (kAux) {
-              const float tt = __fmul_rn(T[k], __fsub_rn(1.0f, alpha));
-              const bool ok = !done[k] && pw <= 0.0f && alpha >= 1.0f / 255.0f;
-              const bool fin = ok && tt < 0.0001f;
-              const bool upd = ok && !fin;
-              const float w = upd ? __fmul_rn(alpha, T[k]) : 0.0f;
-              C0[k] = __fmaf_rn(rgb.x, w, C0[k]);
-              C1[k] = __fmaf_rn(rgb.y, w, C1[k]);
-              C2[k] = __fmaf_rn(rgb.z, w, C2[k]);
               Z[k] = __fmaf_rn(cz.y, w, Z[k]);
-              bl += upd ? 1u : 0u;
-              T[k] = upd ? tt : T[k];
-              last[k] = upd ? pos : last[k];
-              stop[k] = fin ? pos : stop[k];
-              done[k] = done[k] || fin;
+              note(k, a, tt, pos);
             } else {
-              const float a = (pw <= 0.0f && alpha >= 1.0f / 255.0f) ? alpha : 0.0f;
-              const float tt = __fmul_rn(T[k], __fsub_rn(1.0f, a));
-              const bool fin = tt < 0.0001f;   // this Gaussian would end the pixel, or it ended
-              const float w = fin ? 0.0f : __fmul_rn(a, T[k]);
-              C0[k] = __fmaf_rn(rgb.x, w, C0[k]);
-              C1[k] = __fmaf_rn(rgb.y, w, C1[k]);
-              C2[k] = __fmaf_rn(rgb.z, w, C2[k]);
               T[k] = fin ? 0.0f : tt;
             }
           }
@@ -477,7 +436,8 @@ __device__ __forceinline__ void render_pixels(ItemSmem<kMult> &sm, const Composi
   for (int k = 0; k < P; ++k) {
     if (!inside[k]) continue;
     if (kAux) {
-      if (!done[k]) stop[k] = range.y - range.x;
+      if (T[k] > 0.0f) stop[k] = range.y - range.x;
+      T[k] = fabsf(T[k]);
       ev += stop[k];
     }
     const size_t pix = ((size_t)eye * p.height + (size_t)fpy[k]) * p.width + (size_t)fpx[k];
@@ -490,6 +450,7 @@ __device__ __forceinline__ void render_pixels(ItemSmem<kMult> &sm, const Composi
       depth[pix] = Z[k];
     }
   }
+  bl += blended;
   if (inherit && inside[0]) {
     for (int L = hi; L < 4; ++L) {
       const int x = px0 + label_dx(L), y = py0 + label_dy(L);
@@ -576,7 +537,7 @@ __device__ __forceinline__ LanePixels<Q> pixels16(const CompositeParams &p, int 
 }
 
 template <bool kAux, int kMult, int kShape>
-__global__ void __launch_bounds__(kHalfThreads, kAux ? 6 : 7)
+__global__ void __launch_bounds__(kHalfThreads, kAux ? (kShape == kTile32 ? 6 : 5) : 7)
 composite_px_kernel(const CompositeParams *__restrict__ pp, const float *__restrict__ rec, int n,
                     const uint2 *__restrict__ ranges, const uint32_t *__restrict__ kept,
                     const uint32_t *__restrict__ vals, const uint32_t *__restrict__ items,
