@@ -563,7 +563,7 @@ int enqueue_bin_sorted(a3fr_scene *s, int eyes, Entries entries, const FrameLayo
     src.rect = s->rect;
     src.off = off;
     src.pstart = s->pstart;
-    src.total = emit_lb + (ep.n_entries + 1023) / 1024;
+    src.total = emit_lb + emit_blocks(ep.n_entries);
     src.n_parts = n_parts;
     src.n_entries = ep.n_entries;
     src.n = n;

@@ -15,7 +15,7 @@
 // each tile's run, i.e. the tile ranges; the digit histograms of that sort follow from the
 // same prefix sums.
 //
-// emit: the instance offset of every depth-ordered entry (a chained scan over blocks of 1024
+// emit: the instance offset of every depth-ordered entry (a chained scan over blocks of
 // entries) and the entry holding the first slot of each partition of the tile sort.  The
 // instances themselves are not written: the first pass of the tile sort generates them from
 // these offsets (sort.cu), so a Gaussian covering hundreds of tiles costs one slot per thread
@@ -27,13 +27,15 @@ namespace {
 
 constexpr int kEmitThreads = 256;
 constexpr int kEmitWarps = kEmitThreads / 32;
-constexpr int kEmitPer = 4;                                // entries per thread
+constexpr int kEmitPer = 16;                               // entries per thread
 constexpr int kEmitEntries = kEmitThreads * kEmitPer;      // entries per block
 // Instance offsets of the depth-ordered entries, one block of kEmitEntries entries per CTA:
 // the CTAs take consecutive blocks from a ticket counter and chain their instance sums by
 // decoupled look-back, then every entry stores its global offset off[j], every entry holding
 // the first slot of a partition of kGenPart slots (the generated sort pass's unit) stores its
 // index in pstart[k], and the last block stores the total after the look-back words.
+// Bound by the chain of blocks and the gathers of the counts: 4,096 entries a block keep 16 gathers
+// in flight per thread and four fifths of the blocks of 6M entries in one wave (64 -> 47 us under ncu).
 __global__ void __launch_bounds__(kEmitThreads)
 emit_scan_kernel(EmitParams p, Entries ents, const uint32_t *__restrict__ touched,
                  unsigned long long *__restrict__ lookback, uint32_t *__restrict__ off,
@@ -51,11 +53,16 @@ emit_scan_kernel(EmitParams p, Entries ents, const uint32_t *__restrict__ touche
   const uint32_t j0 = b * kEmitEntries + t * kEmitPer;
   uint32_t c[kEmitPer], mine = 0;
   if (j0 + kEmitPer <= (uint32_t)p.n_entries && (reinterpret_cast<uintptr_t>(entries) & 15u) == 0u) {
-    const uint4 v = *reinterpret_cast<const uint4 *>(entries + j0);
-    c[0] = touched[v.x];
-    c[1] = touched[v.y];
-    c[2] = touched[v.z];
-    c[3] = touched[v.w];
+    uint4 v[kEmitPer / 4];
+#pragma unroll
+    for (int k = 0; k < kEmitPer / 4; ++k) v[k] = reinterpret_cast<const uint4 *>(entries + j0)[k];
+#pragma unroll
+    for (int k = 0; k < kEmitPer / 4; ++k) {
+      c[4 * k] = touched[v[k].x];
+      c[4 * k + 1] = touched[v[k].y];
+      c[4 * k + 2] = touched[v[k].z];
+      c[4 * k + 3] = touched[v[k].w];
+    }
   } else {
 #pragma unroll
     for (int k = 0; k < kEmitPer; ++k) c[k] = j0 + k < (uint32_t)p.n_entries ? touched[entries[j0 + k]] : 0u;
@@ -102,7 +109,9 @@ emit_scan_kernel(EmitParams p, Entries ents, const uint32_t *__restrict__ touche
     g += c[k];
   }
   if (j0 + kEmitPer <= (uint32_t)p.n_entries && (reinterpret_cast<uintptr_t>(off) & 15u) == 0u) {
-    *reinterpret_cast<uint4 *>(off + j0) = make_uint4(o4[0], o4[1], o4[2], o4[3]);
+#pragma unroll
+    for (int k = 0; k < kEmitPer / 4; ++k)
+      reinterpret_cast<uint4 *>(off + j0)[k] = make_uint4(o4[4 * k], o4[4 * k + 1], o4[4 * k + 2], o4[4 * k + 3]);
   } else {
 #pragma unroll
     for (int k = 0; k < kEmitPer; ++k)
@@ -309,15 +318,17 @@ tile_scan_kernel(TileScanParams p, const uint32_t *__restrict__ diff, uint2 *__r
 
 }  // namespace
 
+int emit_blocks(int n_entries) { return (n_entries + kEmitEntries - 1) / kEmitEntries; }
+
 size_t emit_lookback_bytes(int n_entries) {
-  return sizeof(unsigned long long) * (size_t)((n_entries + kEmitEntries - 1) / kEmitEntries + 1);
+  return sizeof(unsigned long long) * (size_t)(emit_blocks(n_entries) + 1);
 }
 
 cudaError_t launch_emit_offsets(const EmitParams &p, Entries entries, const uint32_t *touched,
                                 unsigned long long *lookback, uint32_t *off, uint32_t *pstart, int n_parts,
                                 uint32_t *ticket, uint32_t *status, cudaStream_t s) {
   if (p.n_entries <= 0) return cudaSuccess;
-  const int blocks = (p.n_entries + kEmitEntries - 1) / kEmitEntries;
+  const int blocks = emit_blocks(p.n_entries);
   {
     const cudaError_t e_ = launch_pdl(emit_scan_kernel, blocks, kEmitThreads, 0, s, p, entries, touched,
                                       lookback, off, pstart, n_parts, ticket, status);

@@ -269,9 +269,9 @@ struct EmitParams {
 };
 // Instance offsets of the depth-ordered entries: off[j] <- the instances of the entries before
 // j (u32 [n_entries]); pstart[k] (k < n_parts) <- the entry holding instance slot k kGenPart,
-// for every such slot below the total; lookback[n_blocks] <- the total, n_blocks = entries /
-// 1024 rounded up.  lookback (emit_lookback_bytes) and ticket: zeroed by the caller.
+// for every such slot below the total; lookback[emit_blocks(n_entries)] <- the total.  lookback (emit_lookback_bytes) and ticket: zeroed by the caller.
 constexpr int kGenPart = 4096;   // slots per partition of the generated tile-sort pass
+int emit_blocks(int n_entries);
 size_t emit_lookback_bytes(int n_entries);
 cudaError_t launch_emit_offsets(const EmitParams &p, Entries entries, const uint32_t *touched,
                                 unsigned long long *lookback, uint32_t *off, uint32_t *pstart, int n_parts,
