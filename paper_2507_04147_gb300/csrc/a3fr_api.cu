@@ -73,7 +73,7 @@ struct a3fr_scene {
   uint32_t *tile_lb = nullptr;               // the tile sort's look-back (capacity-sized)
   uint32_t *pstart = nullptr;                // first entry of every tile-sort partition
   size_t tile_lb_bytes = 0;
-  uint32_t *plan = nullptr;                  // tiles bucketed by level (foveated composite)
+  uint32_t *plan = nullptr;                  // the composite's work items (plan_bytes)
   uint8_t *levels = nullptr;
   float *t_final = nullptr;
   uint32_t *n_contrib = nullptr;

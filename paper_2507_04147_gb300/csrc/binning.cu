@@ -18,8 +18,9 @@
 //               start overwrites h.  One CTA per 32 tiles; the CTAs chain their sums by a
 //               decoupled look-back (bounded waits, like the sort's).
 //  bin_emit     One warp per (chunk, band of tile rows) walks the chunk's instances in its
-//               band in entry order, 32 at a time (lane = instance).  A lane's slot is the tile's cursor plus the number
-//               of lower lanes with the same tile; the highest of them advances the cursor.
+//               band in entry order, 32 at a time (lane = instance).  A lane's slot is the tile's
+//               cursor plus the number of lower lanes with the same tile; the highest of them
+//               advances the cursor.
 //               Every tile's instances land in entry (= depth) order, the same on every run.
 //
 // Instances whose slot is at or past the capacity are dropped (the render raises the
@@ -400,7 +401,8 @@ BinParams bin_params(int n_eyes, int n, int tiles_x, int tiles_y, uint32_t capac
   p.row = (int)((n_ranges + 3) / 4 * 4);
   // bin_emit: one warp per (chunk, band of tile rows); a band holds at most kBandTiles tiles
   // (whole rows, at least one), so a warp's cursor table stays small however many tiles the
-  // render has and many warps fit on an SM
+  // render has and many warps fit on an SM.  1M Gaussians in 4,096 tiles: one band 86 us, two 76;
+  // in 8,160: two (halves) 194, three (the middle one holds most) 262, four 218.
   const int rows = n_eyes * tiles_y;
   // two bands (an eye each, or the image's halves: views are densest in the middle), more while a
   // band's tables are too large

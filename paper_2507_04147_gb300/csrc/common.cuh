@@ -358,11 +358,9 @@ size_t plan_bytes(int n_ranges);
 // the first round of a frame renders every tile at level `uniform` from label 0 and sets cur;
 // a later round (round != nullptr) renders from cur up to the level of its gaze and radii,
 // stores only those pixels, and raises cur; p.full renders every tile at level 4.  Ranges
-// are clamped to kept[0] (the instances the sort kept).  32-pixel tiles: the plan cuts tiles
-// into work items (plan32) and one persistent launch renders them all, heaviest first;
-// 16-pixel tiles: the plan buckets tiles by label count (none for p.full) and one launch
-// packs them into CTAs.  p (host copy) decides the launch shape; the kernels read p_dev (the
-// same values).  *kernels (optional) receives the number of kernels launched.
+// are clamped to kept[0] (the instances the sort kept).  The plan lists tiles, or halves of them,
+// as work items and one persistent launch renders them all, heaviest first.  p (host copy) decides
+// the launch shape; the kernels read p_dev (the same values).  *kernels (optional) receives the number of kernels launched.
 cudaError_t launch_composite(const CompositeParams &p, const CompositeParams *p_dev,
                              const float *rec, int n, const uint2 *ranges, const uint32_t *kept,
                              const uint32_t *vals, const float *gaze, const RoundPlan *round,

@@ -1,26 +1,18 @@
 // composite.cu -- foveated front-to-back compositing of every tile of every eye (Sec. 2.3
 // "Rasterization"; Sec. 3.4 AMR; Sec. 3.5 implementation details).
 //
-// Work is split the way the paper splits a tile: one group per 2x2-block label (TL 1,
-// BR 2, TR 3, BL 4), and a level-k tile runs only the groups of labels 1..k.  Here a group
-// is two warps: a 16x16 tile has 64 pixels per label, one per lane.
+// The paper splits a tile into one group per label of its 2x2 blocks (TL 1, BR 2, TR 3, BL 4), and a
+// level-k tile runs only the groups of labels 1..k.  Here a label's pixels are assigned to lanes or
+// not at all.  plan_kernel computes every tile's level from the gaze in the device mailbox (Eq. 1: the
+// distance from the gaze to the tile's nearest pixel centre against r_k = f tan(theta_k)) and lists
+// the tiles, or halves of them, as work items by the length of their Gaussian lists; composite_px is
+// one persistent launch that takes the items, the heaviest first.
 //
-// fovea_plan computes every tile's level from the gaze in the device mailbox (Eq. 1: the
-// distance from the gaze to the tile's nearest pixel centre against r_k = f tan(theta_k))
-// and buckets the tiles by level.  composite then packs 8-warp CTAs so that no warp idles:
-//   level 4: one tile per CTA, the CTA stages each batch of Gaussians together;
-//   level 3: one tile per CTA, the last two warps only help staging;
-//   level 2: two tiles per CTA, each half stages its own tile (named barrier);
-//   level 1: four tiles per CTA, each warp pair stages its own tile (named barrier).
-// A full-resolution render skips the plan: every tile is a level-4 CTA.
-//
-// Per batch, the staging threads gather the tile's next Gaussians (indices from the
-// sorted values) into shared memory; each warp then blends them front to back with the
-// 1/255 skip, the 0.99 clamp and the 1e-4 transmittance stop; the staging group stops when
-// all its pixels are done.  The exp of the falloff uses the MUFU ex2 unit with log2(e)
-// folded into the conic.  The blend is branch-free (predicated updates), so a warp whose
-// lanes disagree on the accept test does not run both sides.  Label-1 warps also write the
-// inherited pixels of their blocks.
+// Per batch, a CTA gathers the tile's next Gaussians (indices from the sorted values) into shared
+// memory; each warp lists those that reach its patch and blends them front to back with the 1/255
+// skip, the 0.99 clamp and the 1e-4 transmittance stop, until all its pixels are done.  The exp of
+// the falloff uses the MUFU ex2 unit with log2(e) folded into the conic.  The blend is branch-free,
+// so a warp whose lanes disagree on the accept test does not run both sides.
 #include <algorithm>
 
 #include "blend.cuh"
@@ -208,7 +200,7 @@ plan_kernel(const CompositeParams *__restrict__ pp, const float *__restrict__ ga
 enum : int { kTile32 = 0, kTile16 = 1, kTile16Split = 2 };
 constexpr int kHalfThreads = 128;
 constexpr int kBatch = 256;   // Gaussians staged per batch (times the staging multiple)
-// 16-pixel tiles are split in halves up to this many tiles per SM (of about 9 CTAs resident).  Whole
+// 16-pixel tiles are split in halves up to this many tiles per SM (of 7 CTAs resident).  Whole
 // render, split / not: 256 tiles 163 / 188 us, 825 tiles (training step) 420 / 451 us, 4,096 tiles
 // (training step) 896 / 889 us, 5,670 tiles 241 / 227 us, 8,160 tiles 616 / 567 us.
 constexpr int kSplitTilesPerSm = 16;
