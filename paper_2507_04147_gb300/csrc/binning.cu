@@ -37,7 +37,7 @@ constexpr int kPlanEntries = kPlanThreads * kPlanPer;
 constexpr int kOffsetThreads = 1024;
 constexpr int kMaxChunks = kBinMaxChunks;
 constexpr int kSegUnroll = 16;              // bin_offsets loads in flight per thread
-constexpr int kBandTiles = 6400;            // most tiles of a bin_emit band (32 KB of cursors and tags)
+constexpr int kBandTiles = 2560;            // most tiles of a bin_emit band (12.8 KB of cursors and tags)
 constexpr long long kMaxChunkCells = 24ll << 20;   // bound on C * tiles (u32 cells of h)
 
 // Inclusive scan of one value per lane across the warp.
@@ -232,10 +232,15 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(gmem) : "memory");
+}
 
-// One warp (CTA) per (chunk, band): blockIdx.x = chunk * n_bands + band, the band being the
-// tile rows [R0, R1) (row index eye * tiles_y + y), i.e. the contiguous tiles [R0 tiles_x,
-// R1 tiles_x).  The warp walks the chunk's entries 32 at a time (lane = entry), scans their
+// One warp (CTA) per (chunk, band): blockIdx.x = chunk * n_bands + band, the band being
+// consecutive tile rows (row index eye * tiles_y + y) or, with more than two bands, every
+// n_bands-th row from row `band` on.
+// The warp walks the chunk's entries 32 at a time (lane = entry), scans their
 // instance counts inside the band and writes a record (first instance, first tile, width, Gaussian)
 // of each entry that has any; then it takes the instances 32 at a time (lane = instance: full warps
 // whatever the rectangle sizes).  An instance's entry is the number of first instances at or before
@@ -260,17 +265,25 @@ bin_emit_kernel(BinParams p, Entries ents, const ushort4 *__restrict__ rect,
   __shared__ uint4 s_rec[32];
   const int lane = threadIdx.x;
   const int chunk = blockIdx.x / p.n_bands, band = blockIdx.x - chunk * p.n_bands;
-  const int R0 = band * p.band_rows, R1 = min(p.n_eyes * p.tiles_y, R0 + p.band_rows);
-  // the band's tiles [R0 tiles_x, R1 tiles_x) of the chunk's row of h, copied from the
-  // 16-byte boundary at or below its start; s_cur[t] is the cursor of band tile t
-  const int t0 = R0 * p.tiles_x, a0 = t0 & ~3, a1 = min(p.row, (R1 * p.tiles_x + 3) & ~3);
-  uint32_t *s_cur = s_dyn + (t0 - a0);
+  // band row l is tile row R0 + (l << shift), l < n_rows; s_cur[l tiles_x + x] is the cursor of
+  // its tile x, from the chunk's row of h: consecutive rows in 16-byte pieces from the boundary at
+  // or below their start
+  const int shift = p.n_bands > 2 ? 31 - __clz(p.n_bands) : 0;
+  const int rows = p.n_eyes * p.tiles_y, R0 = shift ? band : band * p.band_rows;
+  const int n_rows = shift ? (rows - band + p.n_bands - 1) >> shift : min(p.band_rows, rows - R0);
+  const int t0 = R0 * p.tiles_x;
+  uint32_t *s_cur = s_dyn + (shift ? 0 : t0 & 3);
   uint8_t *s_tag = reinterpret_cast<uint8_t *>(s_dyn + p.band_rows * p.tiles_x + 8);   // last lane at a band tile
-  {
-    const uint32_t *hb = h + (size_t)chunk * p.row;
+  const uint32_t *hb = h + (size_t)chunk * p.row;
+  if (shift == 0) {
+    const int a0 = t0 & ~3, a1 = min(p.row, (t0 + n_rows * p.tiles_x + 3) & ~3);
     for (int i = a0 + lane * 4; i < a1; i += 128) cp_async16(s_dyn + (i - a0), hb + i);
-    asm volatile("cp.async.commit_group;" ::: "memory");
+  } else {
+    for (int l = 0; l < n_rows; ++l)
+      for (int x = lane; x < p.tiles_x; x += 32)
+        cp_async4(s_cur + l * p.tiles_x + x, hb + (R0 + (l << shift)) * p.tiles_x + x);
   }
+  asm volatile("cp.async.commit_group;" ::: "memory");
   const unsigned below = (1u << lane) - 1u, upto = below | (1u << lane);
   const int j0 = (int)bounds[chunk], j1 = (int)bounds[chunk + 1];
   const ushort4 none = make_ushort4(0, 0, 0, 0);
@@ -290,9 +303,11 @@ bin_emit_kernel(BinParams p, Entries ents, const ushort4 *__restrict__ rect,
     }
     const uint32_t w = rc.z > rc.x ? (uint32_t)(rc.z - rc.x) : 0u;
     const int eye = v >= (uint32_t)p.n ? 1 : 0;
-    // the rectangle's rows inside the band
-    const int row0 = max(R0, eye * p.tiles_y + (int)rc.y);
-    const int row1 = min(R1, eye * p.tiles_y + (int)rc.w);
+    // the rectangle's band rows [row0, row1): the band's rows at or past tile row y are those from
+    // ceil((y - R0) / 2^shift) on
+    const int up = eye * p.tiles_y - R0 + (1 << shift) - 1;
+    const int row0 = max(0, up + (int)rc.y) >> shift;
+    const int row1 = min(n_rows, max(0, up + (int)rc.w) >> shift);
     const uint32_t cnt = (b + lane < j1 && row1 > row0) ? w * (uint32_t)(row1 - row0) : 0u;
     const uint32_t incl = warp_incl_scan(cnt, lane);
     const uint32_t first = incl - cnt;
@@ -301,7 +316,7 @@ bin_emit_kernel(BinParams p, Entries ents, const ushort4 *__restrict__ rect,
     if (total == 0u) continue;
     if (cnt > 0u)
       s_rec[__popc(some & below)] =
-          make_uint4(first, (uint32_t)((row0 - R0) * p.tiles_x + (int)rc.x) | (w << 16), __float_as_uint(__frcp_rn((float)w)),
+          make_uint4(first, (uint32_t)(row0 * p.tiles_x + (int)rc.x) | (w << 16), __float_as_uint(__frcp_rn((float)w)),
                      v - (uint32_t)eye * (uint32_t)p.n);
     __syncwarp();
     uint32_t before = 0;   // entries whose first instance lies before the next instances to expand
@@ -399,18 +414,19 @@ BinParams bin_params(int n_eyes, int n, int tiles_x, int tiles_y, uint32_t capac
   p.capacity = capacity;
   const long long n_ranges = (long long)n_eyes * p.n_tiles;
   p.row = (int)((n_ranges + 3) / 4 * 4);
-  // bin_emit: one warp per (chunk, band of tile rows); a band holds at most kBandTiles tiles
-  // (whole rows, at least one), so a warp's cursor table stays small however many tiles the
-  // render has and many warps fit on an SM.  1M Gaussians in 4,096 tiles: one band 86 us, two 76;
-  // in 8,160: two (halves) 194, three (the middle one holds most) 262, four 218.
+  // bin_emit: one warp per (chunk, band of tile rows).  Two bands of consecutive rows (an eye each,
+  // or the image's halves), which most rectangles fall into one of, while such a band holds at most
+  // kBandTiles tiles; past that 4, 8, ... bands for small tables, so that many warps fit on an SM,
+  // with interleaved rows: views are densest in the middle.  1M Gaussians in 4,096 tiles: one band
+  // 86 us, two 76, two interleaved 80; in 8,160: two 195, three consecutive 262 (the middle one
+  // holds most), four 218, four interleaved 178, eight 189.
   const int rows = n_eyes * tiles_y;
-  // two bands (an eye each, or the image's halves: views are densest in the middle), more while a
-  // band's tables are too large
-  p.n_bands = 2;
-  while (p.n_bands < rows && (long long)((rows + p.n_bands - 1) / p.n_bands) * tiles_x > kBandTiles) p.n_bands *= 2;
-  if (p.n_bands > rows) p.n_bands = rows > 0 ? rows : 1;
+  p.n_bands = rows >= 2 ? 2 : 1;
+  if (rows > 2 && (long long)((rows + 1) / 2) * tiles_x > kBandTiles) {
+    p.n_bands = 4;
+    while (p.n_bands < rows && (long long)((rows + p.n_bands - 1) / p.n_bands) * tiles_x > kBandTiles) p.n_bands *= 2;
+  }
   p.band_rows = rows > 0 ? (rows + p.n_bands - 1) / p.n_bands : 1;
-  p.n_bands = rows > 0 ? (rows + p.band_rows - 1) / p.band_rows : 1;
   // chunks: enough (chunk, band) warps to fill the device (as many as fit at once), at
   // least 256 entries each, at most kMaxChunks and kMaxChunkCells cells of h
   int dev = 0, sms = 152;

@@ -1,6 +1,6 @@
 """Direct placement against the sort-based binning: the same keys, values and tile ranges, bit for bit,
 where the direct one's bands and steps have their edges -- one row of tiles, fewer rows than bands, odd
-rows over two eyes, the most tiles AUTO gives it (four bands), Gaussians that cover every tile, tiles
+rows over two eyes, more than two bands (interleaved rows), Gaussians that cover every tile, tiles
 that several Gaussians of one step share, and a capacity that cuts the lists off."""
 import dataclasses
 
@@ -18,7 +18,9 @@ pytestmark = pytest.mark.gpu
     (16, 700, 2, 32, 2_000, -2.0, 0),       # one column, 2 x 22 rows
     (40, 40, 1, 16, 5_000, -1.0, 0),        # nine tiles: every step shares tiles
     (517, 389, 2, 16, 4_001, -3.5, 0),      # odd rows per eye
-    (2048, 2048, 1, 16, 20_000, -4.0, 0),   # 16,384 tiles, four bands
+    (2048, 2048, 1, 16, 20_000, -4.0, 0),   # 16,384 tiles, the most AUTO gives it: eight bands
+    (1003, 717, 2, 16, 4_003, -3.0, 0),     # 2 x 45 rows in four bands, one of 22 rows
+    (16_384, 80, 1, 16, 3_000, -2.0, 0),    # five rows of the widest view in four bands
     (640, 480, 2, 16, 300, 1.5, 0),         # Gaussians over the whole image
     (517, 389, 1, 16, 4_001, -3.5, 5_000),  # capacity reached
 ])
