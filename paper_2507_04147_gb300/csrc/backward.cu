@@ -18,6 +18,8 @@
 // -> (3-D covariance, Jacobian) -> camera-space position -> mean; 3-D covariance ->
 // scales (through exp) and rotation -> quaternion (through the normalisation); opacity
 // through the sigmoid; colour -> SH coefficients and, through the view direction, mean.
+#include <type_traits>
+
 #include "blend.cuh"
 #include "common.cuh"
 #include "stage.cuh"
@@ -35,6 +37,7 @@ constexpr int kPreBwdCtas = 6;           // CTAs per SM
 // not, 825 quadrants 102 / 145 us, 4,096 quadrants 160 / 146 us (ncu, before the first-order sums
 // were formed per pixel).
 constexpr int kSplitQuadsPerSm = 16;
+constexpr float kTame = 1e15f;           // a few products of two such values are far from overflow
 
 // Where the sums of (eye, Gaussian) entry q of n_entries lie: [n_entries][8] -- the five of p,
 // dopacity, dr, dg (one 32-byte sector) -- then [n_entries] db.
@@ -45,8 +48,11 @@ __device__ __forceinline__ float *sum9(float *g2d, size_t q, size_t n_entries) {
 // label pairs) or of 8 x 4 (Q = 1: 4 x 2 blocks times four labels); per batch it lists the
 // Gaussians that can reach alpha = 1/255 in its patch (falloff_reaches: the others contribute to no
 // pixel of it) and walks only those, two at a time, so that the warp sums of one overlap the
-// other's.  The sums of a batch meet in shared memory, one row per warp and Gaussian, and leave as
-// one reduction per value, Gaussian and quadrant.
+// other's.  A pixel that a listed Gaussian does not touch takes alpha 0 through the same products,
+// which is exact while they are finite; a CTA with an image gradient or a colour that is not below kTame
+// skips such pixels instead, so that a NaN or an infinity reaches only the Gaussians blended at its
+// pixels.  The sums of a batch meet in shared memory, one row per warp and Gaussian, and
+// leave as one reduction per value, Gaussian and quadrant.
 // Bound by issue, and by the longest list's chain on small images.  1M Gaussians at 1024 x 1024 (ncu):
 // 281 us with every warp (16 x 2 pixels) walking the whole list and adding its own nine sums to
 // memory, 154 us now; 50k at 517 x 389: 247, 106 us.
@@ -70,6 +76,8 @@ composite_backward_kernel(BackwardParams p, const float *__restrict__ rec, const
   __shared__ uint32_t s_mask[W][kBatch / 32];   // slots with sums of this warp
   __shared__ float s_sum[W][kBatch + 1][kG2];
   __shared__ uint32_t s_max[W];
+  __shared__ __align__(16) uint32_t s_wild[4];   // 1: a pixel of the warp, or a record it has staged, is not below kTame
+  static_assert(W == 4, "s_wild is read as one vector");
 
   const int qn = p.tile / kTile, parts = Q == 2 ? 1 : 2;
   const int gtile = blockIdx.x / (qn * qn * parts);
@@ -120,12 +128,20 @@ composite_backward_kernel(BackwardParams p, const float *__restrict__ rec, const
       }
     }
   }
+  bool wild_px = false;
+#pragma unroll
+  for (int k = 0; k < Q; ++k)
+    wild_px = wild_px || !(fabsf(g[k][0]) + fabsf(g[k][1]) + fabsf(g[k][2]) <= kTame);
+  wild_px = __any_sync(0xffffffffu, wild_px);
   // the deepest last contributor bounds the walk: the warp's for its lists, the CTA's for the batches
   uint32_t wlast = last[0];
   if (Q == 2) wlast = max(wlast, last[Q - 1]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) wlast = max(wlast, __shfl_xor_sync(0xffffffffu, wlast, o));
-  if (lane == 0) s_max[warp] = wlast;
+  if (lane == 0) {
+    s_max[warp] = wlast;
+    s_wild[warp] = wild_px ? 1u : 0u;
+  }
   if (t == 0) {
     s_geo[kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     s_crg[kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -140,6 +156,106 @@ composite_backward_kernel(BackwardParams p, const float *__restrict__ rec, const
   const float *rec_eye = rec + (size_t)eye * p.n * kRec;
   const size_t n_entries = (size_t)p.n_eyes * p.n, q0 = (size_t)eye * p.n;
 
+  // the nine sums of the Gaussian in slot e over this lane's pixels, and the pixels' state behind it
+  auto evaluate = [&](int e, int hi, float (&v)[kG2], auto guard) {
+    const float4 geo = s_geo[e], crg = s_crg[e];
+    const float cb = s_b[e];
+    const uint32_t pos = (uint32_t)(hi - e);
+#pragma unroll
+    for (int j = 0; j < kG2; ++j) v[j] = 0.0f;
+    if constexpr (decltype(guard)::value) {
+#pragma unroll
+      for (int k = 0; k < Q; ++k) {
+        const float dx = __fsub_rn(geo.x, fpx[k]), dy = __fsub_rn(geo.y, fpy[k]);
+        const float pw = falloff_log2(geo.z, geo.w, crg.x, dx, dy);
+        const float G = ex2_approx(pw), araw = __fmul_rn(crg.y, G), a = fminf(0.99f, araw);
+        if (!(pos <= last[k] && pw <= 0.0f && a >= 1.0f / 255.0f)) continue;
+        const float om = __fsub_rn(1.0f, a);
+        T[k] = T[k] / om;
+        const float w = a * T[k], cdot = crg.z * g[k][0] + crg.w * g[k][1] + cb * g[k][2];
+        const float dal = T[k] * (cdot - D[k]);
+        D[k] = a * cdot + om * D[k];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v[6 + c] += w * g[k][c];
+        if (!(araw <= 0.99f)) continue;   // the clamp passes no gradient
+        const float dpow = dal * araw;
+        v[0] += dpow * (2.0f * geo.z * dx + geo.w * dy);
+        v[1] += dpow * (2.0f * crg.x * dy + geo.w * dx);
+        v[2] += dpow * dx * dx;
+        v[3] += dpow * dx * dy;
+        v[4] += dpow * dy * dy;
+        v[5] += dal * G;
+      }
+    } else if constexpr (Q == 2) {
+      // both pixels per instruction where the arithmetic is the same
+      const f32x2 dx = f2_add(f2_pack(geo.x, geo.x), f2_pack(-fpx[0], -fpx[Q - 1]));
+      const f32x2 dy = f2_add(f2_pack(geo.y, geo.y), f2_pack(-fpy[0], -fpy[Q - 1]));
+      const f32x2 pw = f2_fma(f2_fma(f2_pack(geo.z, geo.z), dx, f2_mul(f2_pack(geo.w, geo.w), dy)), dx,
+                              f2_mul(f2_mul(f2_pack(crg.x, crg.x), dy), dy));
+      float pw0, pw1, ar0, ar1;
+      f2_unpack(pw, pw0, pw1);
+      const float G0 = ex2_approx(pw0), G1 = ex2_approx(pw1);
+      f2_unpack(f2_mul(f2_pack(crg.y, crg.y), f2_pack(G0, G1)), ar0, ar1);
+      const float al0 = fminf(0.99f, ar0), al1 = fminf(0.99f, ar1);
+      const bool ok0 = pos <= last[0] && pw0 <= 0.0f && al0 >= 1.0f / 255.0f;
+      const bool ok1 = pos <= last[Q - 1] && pw1 <= 0.0f && al1 >= 1.0f / 255.0f;
+      // a pixel this Gaussian does not touch takes alpha 0: T and D keep their bits
+      const float a0 = ok0 ? al0 : 0.0f, a1 = ok1 ? al1 : 0.0f;
+      const bool free0 = ok0 && ar0 <= 0.99f, free1 = ok1 && ar1 <= 0.99f;   // the clamp passes no gradient
+      const f32x2 a2 = f2_pack(a0, a1), om = f2_pack(__fsub_rn(1.0f, a0), __fsub_rn(1.0f, a1));
+      T[0] = T[0] / __fsub_rn(1.0f, a0);   // transmittance in front of this Gaussian
+      T[Q - 1] = T[Q - 1] / __fsub_rn(1.0f, a1);
+      const f32x2 T2 = f2_pack(T[0], T[Q - 1]), D2 = f2_pack(D[0], D[Q - 1]);
+      const f32x2 g0 = f2_pack(g[0][0], g[Q - 1][0]), g1 = f2_pack(g[0][1], g[Q - 1][1]),
+                  g2 = f2_pack(g[0][2], g[Q - 1][2]);
+      const f32x2 w2 = f2_mul(a2, T2);
+      const f32x2 cdot = f2_fma(f2_pack(crg.z, crg.z), g0,
+                                f2_fma(f2_pack(crg.w, crg.w), g1, f2_mul(f2_pack(cb, cb), g2)));
+      const f32x2 dal = f2_mul(T2, f2_fma(D2, f2_pack(-1.0f, -1.0f), cdot));
+      f2_unpack(f2_fma(a2, cdot, f2_mul(om, D2)), D[0], D[Q - 1]);
+      const f32x2 dpow = f2_mul(dal, f2_pack(free0 ? ar0 : 0.0f, free1 ? ar1 : 0.0f));
+      const f32x2 px2 = f2_mul(dpow, dx), py2 = f2_mul(dpow, dy);
+      // 2 A dx + B dy and 2 C dy + B dx per pixel, before the sum: in an elongated Gaussian the
+      // two terms nearly cancel
+      const f32x2 bx = f2_pack(geo.w, geo.w);
+      const float A2 = geo.z + geo.z, C2 = crg.x + crg.x;
+      v[0] = f2_sum(f2_mul(dpow, f2_fma(f2_pack(A2, A2), dx, f2_mul(bx, dy))));
+      v[1] = f2_sum(f2_mul(dpow, f2_fma(f2_pack(C2, C2), dy, f2_mul(bx, dx))));
+      v[2] = f2_sum(f2_mul(px2, dx));
+      v[3] = f2_sum(f2_mul(px2, dy));
+      v[4] = f2_sum(f2_mul(py2, dy));
+      v[5] = f2_sum(f2_mul(dal, f2_pack(free0 ? G0 : 0.0f, free1 ? G1 : 0.0f)));
+      v[6] = f2_sum(f2_mul(w2, g0));
+      v[7] = f2_sum(f2_mul(w2, g1));
+      v[8] = f2_sum(f2_mul(w2, g2));
+    } else {
+      const float dx = __fsub_rn(geo.x, fpx[0]), dy = __fsub_rn(geo.y, fpy[0]);
+      const float pw = falloff_log2(geo.z, geo.w, crg.x, dx, dy);
+      const float G = ex2_approx(pw);
+      const float araw = __fmul_rn(crg.y, G);
+      const float al = fminf(0.99f, araw);
+      const bool ok = pos <= last[0] && pw <= 0.0f && al >= 1.0f / 255.0f;
+      const float a = ok ? al : 0.0f;
+      const bool open = ok && araw <= 0.99f;   // the clamp passes no gradient
+      const float om = __fsub_rn(1.0f, a);
+      T[0] = T[0] / om;   // transmittance in front of this Gaussian
+      const float w = a * T[0];
+      const float cdot = crg.z * g[0][0] + crg.w * g[0][1] + cb * g[0][2];
+      const float dal = T[0] * (cdot - D[0]);
+      D[0] = a * cdot + om * D[0];
+      const float dpow = dal * (open ? araw : 0.0f);
+      v[0] = dpow * (2.0f * geo.z * dx + geo.w * dy);
+      v[1] = dpow * (2.0f * crg.x * dy + geo.w * dx);
+      v[2] = dpow * dx * dx;
+      v[3] = dpow * dx * dy;
+      v[4] = dpow * dy * dy;
+      v[5] = dal * (open ? G : 0.0f);
+      v[6] = w * g[0][0];
+      v[7] = w * g[0][1];
+      v[8] = w * g[0][2];
+    }
+  };
+
   for (int hi = (int)max_last; hi >= 1; hi -= kBatch) {
     const int cnt = min(hi, kBatch);   // slot k: 1-based position hi - k of the tile's list
     __syncthreads();                   // the previous batch's sums have left
@@ -149,12 +265,16 @@ composite_backward_kernel(BackwardParams p, const float *__restrict__ rec, const
       const float4 a = __ldg(r4), b = __ldg(r4 + 1);
       s_geo[t] = make_float4(a.x, a.y, __fmul_rn(-0.5f * kLog2e, a.z), __fmul_rn(-kLog2e, a.w));
       s_crg[t] = make_float4(__fmul_rn(-0.5f * kLog2e, b.x), b.y, b.z, b.w);
-      s_b[t] = __ldg(rec_eye + (size_t)gidx * kRec + 8);
+      const float blue = __ldg(rec_eye + (size_t)gidx * kRec + 8);
+      s_b[t] = blue;
+      if (!(b.z + b.w + blue <= kTame)) s_wild[warp] = 1u;   // stays: D keeps what it has met
       s_gid[t] = gidx;
       s_box[t] = int_box(support_box(a.x, a.y, a.z, a.w, b.x, b.y));
       s_thr[t] = -__log2f(255.0f * b.y) - 0.01f;
     }
     __syncthreads();
+    const uint4 wild4 = *reinterpret_cast<const uint4 *>(s_wild);
+    const bool wild = (wild4.x | wild4.y | wild4.z | wild4.w) != 0u;
     int n_hit = 0;
     for (int base = 0; base < kBatch; base += 32) {
       const int k = base + lane;
@@ -175,108 +295,37 @@ composite_backward_kernel(BackwardParams p, const float *__restrict__ rec, const
     }
     if (lane == 0) s_hits[warp][n_hit] = (uint8_t)kBatch;
     __syncwarp();
-    for (int i = 0; i < n_hit; i += 2) {
-      float v[2][kG2];
+    auto walk = [&](auto guard) {
+      for (int i = 0; i < n_hit; i += 2) {
+        float v[2][kG2];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int e = s_hits[warp][i + u];
-        const float4 geo = s_geo[e], crg = s_crg[e];
-        const float cb = s_b[e];
-        const uint32_t pos = (uint32_t)(hi - e);
+        for (int u = 0; u < 2; ++u) evaluate(s_hits[warp][i + u], hi, v[u], guard);
+        // warp sums by recursive halving: at each of the first four steps a lane keeps half of its
+        // values and sends its partner the other half, so the sixteen cost 8 + 4 + 2 + 1 + 1 shuffles;
+        // lane bit 4 ends as the Gaussian, bits 3..1 as the value; the ninth values 1 + 4
+        float h[8];
+        const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0, b2 = (lane & 4) != 0, b1 = (lane & 2) != 0;
 #pragma unroll
-        for (int j = 0; j < kG2; ++j) v[u][j] = 0.0f;
-        if constexpr (Q == 2) {
-          // both pixels per instruction where the arithmetic is the same
-          const f32x2 dx = f2_add(f2_pack(geo.x, geo.x), f2_pack(-fpx[0], -fpx[Q - 1]));
-          const f32x2 dy = f2_add(f2_pack(geo.y, geo.y), f2_pack(-fpy[0], -fpy[Q - 1]));
-          const f32x2 pw = f2_fma(f2_fma(f2_pack(geo.z, geo.z), dx, f2_mul(f2_pack(geo.w, geo.w), dy)), dx,
-                                  f2_mul(f2_mul(f2_pack(crg.x, crg.x), dy), dy));
-          float pw0, pw1, ar0, ar1;
-          f2_unpack(pw, pw0, pw1);
-          const float G0 = ex2_approx(pw0), G1 = ex2_approx(pw1);
-          f2_unpack(f2_mul(f2_pack(crg.y, crg.y), f2_pack(G0, G1)), ar0, ar1);
-          const float al0 = fminf(0.99f, ar0), al1 = fminf(0.99f, ar1);
-          const bool ok0 = pos <= last[0] && pw0 <= 0.0f && al0 >= 1.0f / 255.0f;
-          const bool ok1 = pos <= last[Q - 1] && pw1 <= 0.0f && al1 >= 1.0f / 255.0f;
-          // a pixel this Gaussian does not touch takes alpha 0: T and D keep their bits
-          const float a0 = ok0 ? al0 : 0.0f, a1 = ok1 ? al1 : 0.0f;
-          const bool free0 = ok0 && ar0 <= 0.99f, free1 = ok1 && ar1 <= 0.99f;   // the clamp passes no gradient
-          const f32x2 a2 = f2_pack(a0, a1), om = f2_pack(__fsub_rn(1.0f, a0), __fsub_rn(1.0f, a1));
-          T[0] = T[0] / __fsub_rn(1.0f, a0);   // transmittance in front of this Gaussian
-          T[Q - 1] = T[Q - 1] / __fsub_rn(1.0f, a1);
-          const f32x2 T2 = f2_pack(T[0], T[Q - 1]), D2 = f2_pack(D[0], D[Q - 1]);
-          const f32x2 g0 = f2_pack(g[0][0], g[Q - 1][0]), g1 = f2_pack(g[0][1], g[Q - 1][1]),
-                      g2 = f2_pack(g[0][2], g[Q - 1][2]);
-          const f32x2 w2 = f2_mul(a2, T2);
-          const f32x2 cdot = f2_fma(f2_pack(crg.z, crg.z), g0,
-                                    f2_fma(f2_pack(crg.w, crg.w), g1, f2_mul(f2_pack(cb, cb), g2)));
-          const f32x2 dal = f2_mul(T2, f2_fma(D2, f2_pack(-1.0f, -1.0f), cdot));
-          f2_unpack(f2_fma(a2, cdot, f2_mul(om, D2)), D[0], D[Q - 1]);
-          const f32x2 dpow = f2_mul(dal, f2_pack(free0 ? ar0 : 0.0f, free1 ? ar1 : 0.0f));
-          const f32x2 px2 = f2_mul(dpow, dx), py2 = f2_mul(dpow, dy);
-          // 2 A dx + B dy and 2 C dy + B dx per pixel, before the sum: in an elongated Gaussian the
-          // two terms nearly cancel
-          const f32x2 bx = f2_pack(geo.w, geo.w);
-          const float A2 = geo.z + geo.z, C2 = crg.x + crg.x;
-          v[u][0] = f2_sum(f2_mul(dpow, f2_fma(f2_pack(A2, A2), dx, f2_mul(bx, dy))));
-          v[u][1] = f2_sum(f2_mul(dpow, f2_fma(f2_pack(C2, C2), dy, f2_mul(bx, dx))));
-          v[u][2] = f2_sum(f2_mul(px2, dx));
-          v[u][3] = f2_sum(f2_mul(px2, dy));
-          v[u][4] = f2_sum(f2_mul(py2, dy));
-          v[u][5] = f2_sum(f2_mul(dal, f2_pack(free0 ? G0 : 0.0f, free1 ? G1 : 0.0f)));
-          v[u][6] = f2_sum(f2_mul(w2, g0));
-          v[u][7] = f2_sum(f2_mul(w2, g1));
-          v[u][8] = f2_sum(f2_mul(w2, g2));
-        } else {
-          const float dx = __fsub_rn(geo.x, fpx[0]), dy = __fsub_rn(geo.y, fpy[0]);
-          const float pw = falloff_log2(geo.z, geo.w, crg.x, dx, dy);
-          const float G = ex2_approx(pw);
-          const float araw = __fmul_rn(crg.y, G);
-          const float al = fminf(0.99f, araw);
-          const bool ok = pos <= last[0] && pw <= 0.0f && al >= 1.0f / 255.0f;
-          const float a = ok ? al : 0.0f;
-          const bool open = ok && araw <= 0.99f;   // the clamp passes no gradient
-          const float om = __fsub_rn(1.0f, a);
-          T[0] = T[0] / om;   // transmittance in front of this Gaussian
-          const float w = a * T[0];
-          const float cdot = crg.z * g[0][0] + crg.w * g[0][1] + cb * g[0][2];
-          const float dal = T[0] * (cdot - D[0]);
-          D[0] = a * cdot + om * D[0];
-          const float dpow = dal * (open ? araw : 0.0f);
-          v[u][0] = dpow * (2.0f * geo.z * dx + geo.w * dy);
-          v[u][1] = dpow * (2.0f * crg.x * dy + geo.w * dx);
-          v[u][2] = dpow * dx * dx;
-          v[u][3] = dpow * dx * dy;
-          v[u][4] = dpow * dy * dy;
-          v[u][5] = dal * (open ? G : 0.0f);
-          v[u][6] = w * g[0][0];
-          v[u][7] = w * g[0][1];
-          v[u][8] = w * g[0][2];
-        }
+        for (int j = 0; j < 8; ++j)
+          h[j] = (b4 ? v[1][j] : v[0][j]) + __shfl_xor_sync(0xffffffffu, b4 ? v[0][j] : v[1][j], 16);
+        float h9 = (b4 ? v[1][8] : v[0][8]) + __shfl_xor_sync(0xffffffffu, b4 ? v[0][8] : v[1][8], 16);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          h[j] = (b3 ? h[j + 4] : h[j]) + __shfl_xor_sync(0xffffffffu, b3 ? h[j] : h[j + 4], 8);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          h[j] = (b2 ? h[j + 2] : h[j]) + __shfl_xor_sync(0xffffffffu, b2 ? h[j] : h[j + 2], 4);
+        h[0] = (b1 ? h[1] : h[0]) + __shfl_xor_sync(0xffffffffu, b1 ? h[0] : h[1], 2);
+        h[0] += __shfl_xor_sync(0xffffffffu, h[0], 1);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) h9 += __shfl_xor_sync(0xffffffffu, h9, o);
+        float *row = s_sum[warp][s_hits[warp][i + (b4 ? 1 : 0)]];
+        if (!(lane & 1)) row[(lane >> 1) & 7] = h[0];
+        else if ((lane & 15) == 1) row[8] = h9;
       }
-      // warp sums by recursive halving: at each of the first four steps a lane keeps half of its
-      // values and sends its partner the other half, so the sixteen cost 8 + 4 + 2 + 1 + 1 shuffles;
-      // lane bit 4 ends as the Gaussian, bits 3..1 as the value; the ninth values 1 + 4
-      float h[8];
-      const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0, b2 = (lane & 4) != 0, b1 = (lane & 2) != 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        h[j] = (b4 ? v[1][j] : v[0][j]) + __shfl_xor_sync(0xffffffffu, b4 ? v[0][j] : v[1][j], 16);
-      float h9 = (b4 ? v[1][8] : v[0][8]) + __shfl_xor_sync(0xffffffffu, b4 ? v[0][8] : v[1][8], 16);
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        h[j] = (b3 ? h[j + 4] : h[j]) + __shfl_xor_sync(0xffffffffu, b3 ? h[j] : h[j + 4], 8);
-#pragma unroll
-      for (int j = 0; j < 2; ++j)
-        h[j] = (b2 ? h[j + 2] : h[j]) + __shfl_xor_sync(0xffffffffu, b2 ? h[j] : h[j + 2], 4);
-      h[0] = (b1 ? h[1] : h[0]) + __shfl_xor_sync(0xffffffffu, b1 ? h[0] : h[1], 2);
-      h[0] += __shfl_xor_sync(0xffffffffu, h[0], 1);
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) h9 += __shfl_xor_sync(0xffffffffu, h9, o);
-      float *row = s_sum[warp][s_hits[warp][i + (b4 ? 1 : 0)]];
-      if (!(lane & 1)) row[(lane >> 1) & 7] = h[0];
-      else if ((lane & 15) == 1) row[8] = h9;
-    }
+    };
+    if (!wild) walk(std::false_type{});
+    else walk(std::true_type{});
     __syncthreads();
     // the batch's sums over the warps, eight values of a Gaussian to a sector
     for (int e = t; e < cnt * 8; e += kThreads) {
