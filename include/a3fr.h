@@ -228,6 +228,11 @@ int a3fr_run_frame(a3fr_scene *scene, const a3fr_fovea *fovea, const a3fr_rounds
                    const a3fr_frame_driver *driver, float *out_rgb, void *stream,
                    a3fr_frame_result *result);
 
+/* Every round of the scene's last a3fr_run_frame (A3FR mode), also those past the 16 of its result:
+ * *count receives their number, exits and end_us (HOST arrays of cap entries, either may be NULL) the
+ * exit consumed by each of the first cap rounds and its completion time. */
+int a3fr_get_frame_rounds(a3fr_scene *scene, int32_t *exits, double *end_us, int cap, int *count);
+
 /* Graph mode (default off): renders replay two captured CUDA graphs -- the precompute and
  * the composite (foveated or full) -- instead of launching ~20 operations each; the gaze wait
  * sits between them, so the precompute still overlaps the tracker.  Per-render parameters

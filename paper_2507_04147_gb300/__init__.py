@@ -232,8 +232,8 @@ def get_round_status(handle: int) -> dict:
 def run_frame(handle: int, fovea, rounds, predictions, exit_time_us, out_rgb, mode: int = 0,
               load_period_us: float = 0.0, load_factor: float = 1.0, max_rounds: int = 64,
               stream=None) -> dict:
-    """One frame of Algorithm 1 in native code (see a3fr_run_frame).  "exits" is the exit consumed
-    by each of the first 16 rounds and, when there were more, by the last one."""
+    """One frame of Algorithm 1 in native code (see a3fr_run_frame).  "exits" and "round_end_us" have
+    one entry per round: the exit it consumed and its completion time."""
     pred = np.ascontiguousarray(np.asarray(predictions, dtype=np.float32))
     times = np.ascontiguousarray(np.asarray(exit_time_us, dtype=np.float64))
     d = _lib.FrameDriver()
@@ -244,10 +244,15 @@ def run_frame(handle: int, fovea, rounds, predictions, exit_time_us, out_rgb, mo
     _lib.check(_lib.load().a3fr_run_frame(handle, ctypes.byref(fovea), ctypes.byref(rounds),
                                           ctypes.byref(d), _ptr(out_rgb), _stream_ptr(stream),
                                           ctypes.byref(r)), "a3fr_run_frame")
-    k = min(r.rounds, 16)
-    last = [get_round_status(handle)["exit_consumed"]] if r.rounds > 16 else []
+    exits, ends = list(r.exit_per_round[:r.rounds]), list(r.round_end_us[:r.rounds])
+    if r.rounds > len(exits):
+        n = ctypes.c_int()
+        e, t = (ctypes.c_int32 * r.rounds)(), (ctypes.c_double * r.rounds)()
+        _lib.check(_lib.load().a3fr_get_frame_rounds(handle, e, t, r.rounds, ctypes.byref(n)),
+                   "a3fr_get_frame_rounds")
+        exits, ends = list(e[:n.value]), list(t[:n.value])
     return {"latency_us": r.latency_us, "tracker_end_us": r.tracker_end_us, "rounds": r.rounds,
-            "exits": list(r.exit_per_round[:k]) + last, "round_end_us": list(r.round_end_us[:k])}
+            "exits": exits, "round_end_us": ends}
 
 
 def error_string(code: int) -> str:

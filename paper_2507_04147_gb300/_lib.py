@@ -153,6 +153,8 @@ _SIGS = {
     "a3fr_run_frame": ([ctypes.c_void_p, ctypes.POINTER(Fovea), ctypes.POINTER(Rounds),
                         ctypes.POINTER(FrameDriver), ctypes.c_void_p, ctypes.c_void_p,
                         ctypes.POINTER(FrameResult)], ctypes.c_int),
+    "a3fr_get_frame_rounds": ([ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int,
+                               ctypes.POINTER(ctypes.c_int)], ctypes.c_int),
     "a3fr_set_stage_timing": ([ctypes.c_void_p, ctypes.c_int], ctypes.c_int),
     "a3fr_get_stage_times": ([ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p,
                               ctypes.POINTER(ctypes.c_int)], ctypes.c_int),

@@ -145,6 +145,7 @@ struct a3fr_scene {
   uint64_t g_pre_launches = 0, g_fov_launches = 0, g_full_launches = 0;   // kernels in each graph
 
   int batch_mult = 1;                        // Gaussians staged per thread per composite batch
+  std::vector<FrameRound> frame_log;         // see scene_frame_log
 
   // backward: what the last render leaves for it (0 none, 1 full, 2 foveated; keep_aux only)
   int bw_mode = 0;
@@ -827,6 +828,8 @@ int render_round(a3fr_scene *s, float *out, cudaStream_t stream) {
 }  // namespace
 
 int a3fr::scene_eyes(const a3fr_scene *s) { return n_eyes_of(s); }
+
+std::vector<FrameRound> &a3fr::scene_frame_log(a3fr_scene *s) { return s->frame_log; }
 
 bool a3fr::scene_fill_view(a3fr_scene *s, FillView *v) {
   if (!s || !v || s->bw_mode != 2 || s->last_eyes == 0) return false;

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <vector>
 #include <cuda_runtime.h>
 
 namespace a3fr {
@@ -403,6 +404,12 @@ struct a3fr_scene;
 namespace a3fr {
 // Eyes rendered by a scene (eyes with a camera).
 int scene_eyes(const a3fr_scene *s);
+// the rounds of the scene's last a3fr_run_frame
+struct FrameRound {
+  int exit;         // consumed by the round
+  double end_us;    // its completion
+};
+std::vector<FrameRound> &scene_frame_log(a3fr_scene *s);
 
 // What the learned periphery needs from a scene's last foveated render (keep_aux on):
 // its expected depth and tile levels; false when there is no such render.

@@ -14,7 +14,9 @@
 // full-resolution frame without waiting for the tracker.
 #include <atomic>
 #include <chrono>
+#include <new>
 #include <thread>
+#include <vector>
 
 #include "../../include/a3fr.h"
 #include "common.cuh"
@@ -58,6 +60,8 @@ extern "C" int a3fr_run_frame(a3fr_scene *scene, const a3fr_fovea *fovea,
   cudaEvent_t ev;
   if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) return A3FR_ERR_CUDA;
   *result = a3fr_frame_result{};
+  std::vector<a3fr::FrameRound> &log = a3fr::scene_frame_log(scene);
+  log.clear();
   const int eyes = a3fr::scene_eyes(scene);
   if (eyes == 0) {
     cudaEventDestroy(ev);
@@ -120,11 +124,16 @@ extern "C" int a3fr_run_frame(a3fr_scene *scene, const a3fr_fovea *fovea,
       }
       a3fr_round_status rs{};
       a3fr_get_round_status(scene, &rs);
+      const a3fr::FrameRound entry{rs.exit_consumed, us_since(t0)};
       if (result->rounds < 16) {
-        result->exit_per_round[result->rounds] = rs.exit_consumed;
-        result->round_end_us[result->rounds] = us_since(t0);
+        result->exit_per_round[result->rounds] = entry.exit;
+        result->round_end_us[result->rounds] = entry.end_us;
       }
       result->rounds++;
+      try {
+        log.push_back(entry);
+      } catch (const std::bad_alloc &) {   // the frame goes on; the log ends here
+      }
       idle = rs.exit_consumed == last_seen && rs.radius_px[0] == last_r;
       last_seen = rs.exit_consumed;
       last_r = rs.radius_px[0];
@@ -138,4 +147,15 @@ extern "C" int a3fr_run_frame(a3fr_scene *scene, const a3fr_fovea *fovea,
   result->tracker_end_us = us_since(t0);
   cudaEventDestroy(ev);
   return rc;
+}
+
+extern "C" int a3fr_get_frame_rounds(a3fr_scene *scene, int32_t *exits, double *end_us, int cap, int *count) {
+  if (!scene || !count || cap < 0) return A3FR_ERR_INVALID_ARG;
+  const std::vector<a3fr::FrameRound> &log = a3fr::scene_frame_log(scene);
+  *count = (int)log.size();
+  for (int i = 0; i < cap && i < *count; ++i) {
+    if (exits) exits[i] = log[i].exit;
+    if (end_us) end_us[i] = log[i].end_us;
+  }
+  return A3FR_OK;
 }

@@ -198,3 +198,24 @@ def test_stalled_mailbox_write_times_out_and_keeps_the_last_prediction():
     assert s.round_status()["exit_consumed"] == 2
     assert np.array_equal(_levels(s, eyes, n_tiles), np.stack([f.level for f in fr]))
     print("bounded mailbox wait gave up after %.3f s" % waited)
+
+
+@pytest.mark.parametrize("max_rounds", [7, 16, 17, 40])
+def test_native_frame_driver_reports_every_round(max_rounds):
+    """The driver's lists have one entry a round, however many rounds a frame takes: a slow tracker whose
+    first prediction the renderer goes on speculating from (a small step of Eq. 4 takes hundreds of rounds
+    to its maximum), until the bound on the rounds."""
+    import torch
+    scene_np, cams, s, out = _setup()
+    gfv = a3fr.Fovea()
+    expected = [400.0, 120.0, 0.0]
+    preds = np.tile(np.array([[100.0, 84.0]] * len(cams), np.float32), (3, 1, 1))
+    times = [100.0, 300e3, 310e3]      # microseconds: the second prediction after all the rounds
+    r = a3fr.run_frame(s.handle, gfv, a3fr.Rounds(expected, sir=True, sir_step_px=0.25), preds, times, out,
+                       max_rounds=max_rounds, stream=torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    assert r["rounds"] == max_rounds
+    assert r["exits"] == [1] * max_rounds
+    assert len(r["round_end_us"]) == max_rounds
+    assert all(a < b for a, b in zip([times[0]] + r["round_end_us"], r["round_end_us"] + [times[1]]))
+    s.close()
