@@ -257,8 +257,11 @@ int a3fr_set_batch(a3fr_scene *scene, int batch_mult);
  * instance placed at its slot by ordered ranks (no sort over the instances).  SORTED: tile
  * counts, emit of the depth-ordered instances, a stable radix sort by tile.  AUTO (default):
  * DIRECT up to 6,144 tiles over all eyes, and up to 16,384 while tiles x entries (Gaussians times
- * eyes) is at most 1.6e10; SORTED above (where it is faster).  Changing it invalidates the scene's
- * buffers (the next render reallocates); synchronous.  Invalid mode: A3FR_ERR_INVALID_ARG. */
+ * eyes) is at most 1.6e10 and, for two eyes with more than 8,448 tiles, entries at most 450,000;
+ * SORTED above (where it is, within a few percent, the faster).  When the instances exceed the
+ * capacity (A3FR_STATUS_CAPACITY) DIRECT keeps the tile lists up to the capacity and drops the rest;
+ * which instances SORTED keeps is unspecified.  Changing it invalidates the scene's buffers (the next
+ * render reallocates); synchronous.  Invalid mode: A3FR_ERR_INVALID_ARG. */
 #define A3FR_BINNING_AUTO 0
 #define A3FR_BINNING_DIRECT 1
 #define A3FR_BINNING_SORTED 2

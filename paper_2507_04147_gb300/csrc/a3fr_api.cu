@@ -160,16 +160,27 @@ int n_eyes_of(const a3fr_scene *s) { return s->cam_set[1] ? 2 : (s->cam_set[0] ?
 constexpr int kDepthPasses = 4;   // 32-bit depth keys, 8-bit digits
 
 // AUTO binning: direct placement up to kBinDirectMaxTiles tiles (all eyes), and beyond that for up to
-// kBinDirectMaxTilesBig tiles while tiles x entries stays below kBinDirectMaxWork; else the sort-based
+// kBinDirectMaxTilesBig tiles while tiles x entries stays below kBinDirectMaxWork -- with two eyes and
+// more than kBinDirectStereoTiles tiles, up to kBinDirectStereoEntries entries; else the sort-based
 // binning.  Each direct-binning warp walks one chunk of entries serially, and the chunk table
-// (chunks x tiles) caps the chunk count: with many tiles and entries the chains grow and the stable
-// radix sort by tile is faster.  Tile counts to placed instances, direct / sorted (us; uniform scenes):
-// 8,160 tiles 500k entries 147 / 193, 1M 260 / 319, 2M 618 / 578; 16,320 tiles 100k 70 / 97,
-// 1M 303 / 336, 2M 706 / 601; 17,802 tiles 500k 244 / 224; 8,970 tiles 6M (clustered) 726 / 535.
+// (chunks x tiles) caps the chunk count: with many tiles and entries the chains grow, and the stable
+// radix sort by tile, whose time goes with the instances, is faster -- sooner in stereo, where an entry
+// has half the instances of one eye's render of as many tiles.  Tile counts to placed instances,
+// direct / sorted (us; uniform, clustered scene; the lines lie between the two scenes' crossings):
+//   one eye,  8,160 tiles: 1M entries 243 / 290, 162 / 173;  1.5M 365 / 415, 223 / 232;  2M 589 / 542, 288 / 296
+//            14,400:       700k 269 / 324, 179 / 182;  1M 402 / 441, 234 / 236;  1.5M 749 / 632, 337 / 320
+//   two eyes, 8,256:       1M 181 / 209, 132 / 144;  1.5M 249 / 287, 182 / 186;  2M 336 / 364, 242 / 230
+//             8,970:       300k 85 / 94, 77 / 80;  500k 111 / 110, 99 / 82;  1M 181 / 165, 148 / 122
+//            10,260:       400k 107 / 122, 97 / 97;  500k 124 / 138, 111 / 106;  1M 212 / 220, 173 / 148
+//            11,844:       400k 111 / 128, 97 / 99;  500k 132 / 142, 107 / 107;  1M 224 / 226, 176 / 151
+//            16,320:       400k 144 / 165, 117 / 123;  500k 169 / 185, 130 / 128;  700k 220 / 233, 169 / 153
 constexpr long long kBinDirectMaxTiles = 6144, kBinDirectMaxTilesBig = 16384, kBinDirectMaxWork = 16000000000ll;
+constexpr long long kBinDirectStereoTiles = 8448, kBinDirectStereoEntries = 450000;
 
-bool auto_bin_direct(long long tiles, long long entries) {
-  return tiles <= kBinDirectMaxTiles || (tiles <= kBinDirectMaxTilesBig && tiles * entries <= kBinDirectMaxWork);
+bool auto_bin_direct(int eyes, long long tiles, long long entries) {
+  if (tiles <= kBinDirectMaxTiles) return true;
+  if (tiles > kBinDirectMaxTilesBig || tiles * entries > kBinDirectMaxWork) return false;
+  return eyes < 2 || tiles <= kBinDirectStereoTiles || entries <= kBinDirectStereoEntries;
 }
 
 int tile_bits_for(int n_ranges) {
@@ -297,7 +308,7 @@ int ensure_frame_buffers(a3fr_scene *s, int eyes, int W, int H) {
     A3FR_CHECK(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const int tx = (W + tile - 1) / tile, ty = (H + tile - 1) / tile;
     s->sorted_bin = s->binning == A3FR_BINNING_SORTED ||
-                    (s->binning == A3FR_BINNING_AUTO && !auto_bin_direct((long long)eyes * tx * ty, (long long)eyes * n));
+                    (s->binning == A3FR_BINNING_AUTO && !auto_bin_direct(eyes, (long long)eyes * tx * ty, (long long)eyes * n));
     const size_t need = s->sorted_bin ? tile_scan_smem_bytes(eyes, tx, ty) + 9216 : bin_smem_bytes(eyes, tx, ty);
     if (need > (size_t)max_optin) return A3FR_ERR_INVALID_ARG;
   }

@@ -50,3 +50,32 @@ def test_direct_equals_sorted(w, h, eyes, tile, n, log_scale, capacity):
         return
     for a, b in zip(*got):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("w,h,eyes,tile,n,route", [
+    (2064, 2208, 2, 32, 200_000, a3fr.BINNING_DIRECT),   # 8,970 tiles, 400k entries
+    (2064, 2208, 2, 32, 250_000, a3fr.BINNING_SORTED),   # 500k entries
+    (1366, 768, 2, 16, 250_000, a3fr.BINNING_DIRECT),    # 8,256 tiles
+    (2560, 1440, 1, 16, 500_000, a3fr.BINNING_DIRECT),   # 14,400 tiles of one eye
+    (1280, 720, 1, 16, 1_000, a3fr.BINNING_DIRECT),
+    (2576, 2064, 1, 16, 1_000, a3fr.BINNING_SORTED),     # 20,769 tiles
+])
+def test_auto_takes_the_faster_route(w, h, eyes, tile, n, route):
+    """AUTO's route, told by the number of kernels it launches, and its image."""
+    import __graft_entry__
+    __graft_entry__.build()
+    sc = synth.uniform_scene(n, 0, seed=3, log_scale_mean=-5.0)
+    s = a3fr.Scene.from_numpy(sc, tile=tile)
+    for e, c in enumerate(synth.stereo_cameras(w, h) if eyes == 2 else [synth.pinhole_camera(w, h)]):
+        s.set_camera(e, c)
+    launches, images = {}, {}
+    for mode in (a3fr.BINNING_AUTO, a3fr.BINNING_DIRECT, a3fr.BINNING_SORTED):
+        s.set_binning(mode)
+        s.render_full()
+        s.stats(reset=True)
+        images[mode] = s.render_full().clone()
+        launches[mode] = s.stats()["kernel_launches"]
+    s.close()
+    assert launches[a3fr.BINNING_DIRECT] != launches[a3fr.BINNING_SORTED]
+    assert launches[a3fr.BINNING_AUTO] == launches[route]
+    assert (images[a3fr.BINNING_AUTO] == images[route]).all()
