@@ -79,3 +79,37 @@ def test_auto_takes_the_faster_route(w, h, eyes, tile, n, route):
     assert launches[a3fr.BINNING_DIRECT] != launches[a3fr.BINNING_SORTED]
     assert launches[a3fr.BINNING_AUTO] == launches[route]
     assert (images[a3fr.BINNING_AUTO] == images[route]).all()
+
+
+@pytest.mark.parametrize("w,h,eyes,tile,n,log_scale,capacity", [
+    (517, 389, 1, 16, 4_001, -3.5, 5_000),   # two bands
+    (1003, 717, 2, 16, 4_003, -3.0, 30_001),   # 5,670 tiles: four interleaved bands
+    (640, 480, 2, 16, 300, 1.5, 77_777),     # Gaussians over the whole image: the capacity cuts long lists
+])
+def test_direct_below_the_capacity(w, h, eyes, tile, n, log_scale, capacity):
+    """Direct placement with too small a capacity: what lies below it -- values, keys, and the pixels of
+    tiles whose list ends there -- is what an ample one gives, bit for bit."""
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    sc = synth.uniform_scene(n, 0, seed=n, log_scale_mean=log_scale)
+    cams = synth.stereo_cameras(w, h) if eyes == 2 else [synth.pinhole_camera(w, h)]
+    got = []
+    for cap in (0, capacity):
+        s = a3fr.Scene.from_numpy(sc, instance_capacity=cap, tile=tile)
+        s.set_binning(a3fr.BINNING_DIRECT)
+        for e, c in enumerate(cams):
+            s.set_camera(e, c)
+        img = s.render_full().cpu().numpy()
+        assert s.stats()["status"] == (a3fr.STATUS_CAPACITY if cap else 0)
+        got.append([s.buffer(which, dt).cpu().numpy() for which, dt in (
+            (a3fr.BUF_VALUES, torch.int32), (a3fr.BUF_KEYS, torch.int64), (a3fr.BUF_RANGES, torch.int32))] + [img])
+        s.close()
+    (vals, keys, ranges, img), (vals_c, keys_c, ranges_c, img_c) = got
+    assert len(vals) > capacity and len(vals_c) == len(keys_c) == capacity
+    assert np.array_equal(ranges, ranges_c)
+    assert np.array_equal(vals[:capacity], vals_c) and np.array_equal(keys[:capacity], keys_c)
+    whole = (ranges.reshape(eyes, -1, 2)[..., 1] <= capacity).reshape(eyes, (h + tile - 1) // tile, -1)
+    whole = whole.repeat(tile, 1).repeat(tile, 2)[:, :h, :w]
+    assert whole.any() and not whole.all()
+    assert np.array_equal(img[whole], img_c[whole])
