@@ -11,6 +11,7 @@
 #include "common.cuh"
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <new>
 
@@ -1135,7 +1136,8 @@ __global__ void unpack_grads_kernel(GradMap m, const float *__restrict__ scratch
 
 int grid_1d(size_t n) {
   const size_t b = (n + 255) / 256;
-  return (int)(b < 152 * 16 ? (b > 0 ? b : 1) : 152 * 16);
+  const size_t most = 16 * (size_t)sm_count();
+  return (int)(b < most ? (b > 0 ? b : 1) : most);
 }
 
 }  // namespace
@@ -1210,8 +1212,8 @@ cudaError_t conv(const ConvDims &d, const __nv_bfloat16 *X, const __nv_bfloat16 
     attr[dev] = true;
   }
   const int tiles = d.B * ((d.W + kConvTW - 1) / kConvTW) * ((d.H + kConvTH - 1) / kConvTH);
-  return launch_pdl(conv3x3_tc_kernel<CIN, COUT, FLAGS, SRC, DST>, tiles < 152 ? tiles : 152, kConvThreads, smem, s, d,
-                    X, reinterpret_cast<const uint4 *>(W), bias, R, M, Y, status, io);
+  return launch_pdl(conv3x3_tc_kernel<CIN, COUT, FLAGS, SRC, DST>, std::min(tiles, sm_count()), kConvThreads, smem, s,
+                    d, X, reinterpret_cast<const uint4 *>(W), bias, R, M, Y, status, io);
 }
 
 cudaError_t compact_fill(const ConvDims &d, const a3fr_cnn *n, uint32_t *status, cudaStream_t s, const FillIO &io) {
@@ -1225,7 +1227,7 @@ cudaError_t compact_fill(const ConvDims &d, const a3fr_cnn *n, uint32_t *status,
     attr[dev] = true;
   }
   const int tiles = d.B * ((d.W + kCmpTW - 1) / kCmpTW) * ((d.H + kCmpTH - 1) / kCmpTH);
-  const int grid = tiles < 152 * kCmpCtas ? tiles : 152 * kCmpCtas;
+  const int grid = std::min(tiles, sm_count() * kCmpCtas);
   const int A = A3FR_CNN_COMPACT;
   // the per-block layers' weights: the centre tap (4) of their 3x3 packs [tap][cin/8][cout][8]
   const uint4 *w1 = reinterpret_cast<const uint4 *>(n->wf[1] + 4 * 32 * 32);
@@ -1251,8 +1253,8 @@ cudaError_t wgrad(const a3fr_cnn *n, int l, const ConvDims &d, const __nv_bfloat
   }
   const int tiles = d.B * ((d.H + kWgTH - 1) / kWgTH) * ((d.W + kWgTW - 1) / kWgTW);
   float *dW = n->wscratch + scratch_offset(n->arch, l);
-  return launch_pdl(conv3x3_wgrad_tc_kernel<CIN, COUT>, tiles < 152 ? tiles : 152, kWgThreads, smem, s, d, X, dY, dW,
-                    dW + 9 * CIN * COUT, n->status);
+  return launch_pdl(conv3x3_wgrad_tc_kernel<CIN, COUT>, std::min(tiles, sm_count()), kWgThreads, smem, s, d, X, dY,
+                    dW, dW + 9 * CIN * COUT, n->status);
 }
 
 #define CNN_CHECK(call)                                  \

@@ -482,13 +482,6 @@ onesweep_kernel(Src src, K *__restrict__ keys_out, uint32_t *__restrict__ vals_o
   }
 }
 
-int sm_count() {
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess)
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
-}
-
 template <typename K, int KPT, class Src>
 constexpr size_t onesweep_smem() {
   constexpr size_t staging = (sizeof(K) + sizeof(uint32_t)) * kThreads * KPT;
