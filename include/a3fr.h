@@ -103,7 +103,8 @@ typedef struct {
                                    rendered pixel's position in its tile's list where it
                                    stopped (or the list length); counted by renders with
                                    keep_aux on only (0 otherwise) */
-  uint64_t records_staged;      /* Gaussian records staged by tile blocks since the reset */
+  uint64_t records_staged;      /* Gaussian records staged by tile blocks since the reset (a list
+                                   that two half tiles walk counts twice) */
   uint64_t renders;             /* renders since the last reset */
   uint64_t kernel_launches;     /* kernels this library launched since the last reset */
   uint64_t contributions;       /* (pixel, Gaussian) blends since the last reset, counted by
@@ -244,10 +245,10 @@ int a3fr_get_frame_rounds(a3fr_scene *scene, int32_t *exits, double *end_us, int
 int a3fr_set_graph_mode(a3fr_scene *scene, int on);
 
 /* ------------------------------------------------------------------ tiling and tuning
- * Tile size (16 or 32 pixels; the paper tiles 32 x 32, Sec. 3.5): with 32, every label of a
- * tile is its own 256-thread CTA and only the labels a tile's level needs are launched.  The
- * per-thread staging batch (1 or 2 Gaussians per thread per shared-memory batch) trades
- * barrier count for shared memory.  Changing either invalidates the scene's buffers and
+ * Tile size (16 or 32 pixels; the paper tiles 32 x 32, Sec. 3.5): a CTA renders a tile, or half of
+ * one (32-pixel tiles, and 16-pixel tiles where there are few), and only the labels its level
+ * needs.  The staging batch (256 or 512 Gaussians in shared memory at a time, multiple 1 or 2)
+ * trades barrier count for shared memory.  Changing either invalidates the scene's buffers and
  * captured graphs (the next render reallocates); synchronous. */
 int a3fr_set_tile(a3fr_scene *scene, int tile);
 int a3fr_set_batch(a3fr_scene *scene, int batch_mult);

@@ -26,6 +26,7 @@
 // Instances whose slot is at or past the capacity are dropped (the render raises the
 // capacity status and the composite clamps ranges to the instances kept).
 #include "common.cuh"
+#include "stage.cuh"
 
 namespace a3fr {
 namespace {
@@ -228,10 +229,6 @@ bin_offsets_kernel(BinParams p, uint32_t *__restrict__ h, unsigned long long *__
   }
 }
 
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
-}
 __device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(gmem) : "memory");

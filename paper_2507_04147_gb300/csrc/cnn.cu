@@ -231,6 +231,10 @@ struct TileWalk {
 // 131 us with one MMA warp and copies straight to shared memory, 140 us with five CTAs of 128 threads
 // per SM that each loaded, multiplied and stored in turn.  Without it 102 -> 80 us; 16 x 128 x 128
 // pixels 22 -> 15 us.  MMAs of several tiles interleaved in one issue stream: no faster.
+//
+// Twelve accumulators take all 512 columns of an SM's tensor memory (allocations are powers of two), so
+// a kernel of another stream that needs some (a compact fill) shares no SM with this one: its CTA waits
+// in its allocation until this one's ends.
 constexpr int kConvStages = 12;                    // even: see the parities below; 32 accumulator columns each
 constexpr int kConvThreads = 2 * 128 + 2 * 128 + 2 * 32;   // epilogue groups, copying groups, MMA warps
 constexpr int kConvHR = kConvTH + 2, kConvHC = kConvTW + 2;

@@ -68,10 +68,10 @@ __device__ inline unsigned long long block_lookback(unsigned long long *lookback
 
 // Programmatic dependent launch: the kernels of a render run back to back in one stream, each
 // launched with programmatic stream serialisation (launch_pdl), so the next kernel's CTAs can
-// be scheduled while this one's last CTAs finish.  Every such kernel starts with pdl_begin():
-// it lets the next kernel be scheduled once all of its own CTAs have started, then waits until
-// the previous kernel has completed and its writes are visible -- before touching any memory.
-// Both instructions are no-ops in a kernel launched without the attribute.
+// be scheduled while this one's last CTAs finish.  Every such kernel calls pdl_begin() before it
+// touches global memory: it waits until the previous kernel has completed and its writes are visible.
+// None triggers its dependents early, so these are scheduled once all its CTAs have exited or are
+// exiting.  The instruction does nothing in a kernel launched without the attribute.
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

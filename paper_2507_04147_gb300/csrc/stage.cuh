@@ -1,5 +1,5 @@
 // stage.cuh -- staging of a block's slices of the scene arrays in shared memory, shared by the
-// projection and its backward.
+// projection and its backward, and the 16-byte asynchronous copy.
 #pragma once
 
 #include <cuda_runtime.h>
