@@ -55,7 +55,7 @@ __device__ __forceinline__ float *sum9(float *g2d, size_t q, size_t n_entries) {
 // leave as one reduction per value, Gaussian and quadrant.
 // Bound by issue, and by the longest list's chain on small images.  1M Gaussians at 1024 x 1024 (ncu):
 // 281 us with every warp (16 x 2 pixels) walking the whole list and adding its own nine sums to
-// memory, 154 us now; 50k at 517 x 389: 247, 106 us.
+// memory, 152 us now; 50k at 517 x 389: 247, 106 us.
 template <int Q>
 __global__ void __launch_bounds__(kThreads, 6)
 composite_backward_kernel(BackwardParams p, const float *__restrict__ rec, const uint2 *__restrict__ ranges,
